@@ -57,7 +57,7 @@ def sc_kw(n=N3, nz=None):
 
 # Sources that define the FP32 step kernels and their launch (the profiled kernels).
 STEP_KERNEL_SOURCES = ("lbm_lattice.cuh", "lbm_rep.cuh", "lbm_step.cuh", "lbm_step_tma.cuh", "lbm_step_tmac.cuh",
-                       "lbm_step_ring.cuh", "lbm_launch.cuh", "lbm_internal.cuh", "lbm_step_f32.cu")
+                       "lbm_vec.cuh", "lbm_step_pair.cuh", "lbm_launch.cuh", "lbm_internal.cuh", "lbm_step_f32.cu")
 
 
 def csrc_sha256_16():
@@ -255,19 +255,12 @@ def serving_sweep(n_req: int, seed: int = 5):
 
 
 def kernel_label(model: str, precision: int, tiling) -> str:
-    """The step kernel a tiling runs on the 128^3 benchmark lattices (nx / tx <= 8): the
-    ring kernel for 32 x 16 and 64 x 8 tiles, and for 64 x 4 tiles where two of its blocks
-    fit an SM (SC multiphase, or 16-bit storage); the cluster TMA kernel for the other
-    32 x 8, 32 x 4 and 64 x 4 tiles; the generic kernel otherwise.  The label names the
-    tile, whose traffic differs."""
-    tx, ty = int(tiling[0]), int(tiling[1])
+    """The step kernel a tiling runs on the 128^3 benchmark lattices: the pair kernel for the
+    tilings that name a TMA-staged kernel, the generic kernel otherwise."""
     elt = {1: "float", 2: "half", 3: "bf16"}[precision]
     m = "CG" if model == "cg" else "SC-MP"
-    ring = (tx, ty) in ((32, 16), (64, 8)) or ((tx, ty) == (64, 4) and (model == "sc" or precision != 1))
-    if ring and not (model == "cg" and precision == 1 and tx == 64):
-        return f"step_kernel_ring<D3Q19,{elt},{m},{tx}x{ty}>"
-    if (tx, ty) in ((32, 8), (32, 4), (64, 4)):
-        return f"step_kernel_tmac<D3Q19,{elt},{m},{tx}x{ty}>"
+    if (int(tiling[0]), int(tiling[1])) in ((32, 8), (32, 4), (64, 4), (32, 16), (64, 8)):
+        return f"step_kernel_pair<D3Q19,{elt},{m}>"
     return f"step_kernel<D3Q19,{elt},{m}>"
 
 

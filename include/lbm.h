@@ -173,16 +173,14 @@ const char* lbm_status_string(lbm_status s);
  * ceil(nz / tz) chunks of near-equal length, one block per unit (tz must be 1 for D2Q9).
  * tz = 0: a persistent grid of as many blocks as fit on the device looping over the units,
  * with a chunk count chosen from that block count.  Default 32 x 8 x 16.
- * D3Q19 lattices in FP32/FP16/BF16 with nx % 32 == 0 and ny % 8 == 0 run the TMA-staged
- * kernel when tx x ty is 32 x 8 (for nx <= 256 as clusters of nx / 32 blocks that exchange
- * the x-halo in distributed shared memory; the cluster kernel also takes 32 x 4, with two
- * blocks per SM, and 64 x 4 when nx % 64 == 0, in clusters of nx / 64), the generic kernel
- * otherwise.  The ring kernel (the next plane's node state carried in registers, halo
- * columns as asynchronous remote stores) takes the CG and SC-multiphase models without
- * walls or the repulsion force: 32 x 16 and 64 x 8 tiles (one 512-thread block per SM;
- * D3Q19 only; where it does not apply, the step runs 32 x 8 tiles), and 64 x 4 tiles
- * where two of its blocks fit an SM (SC multiphase, or 16-bit storage), in clusters of
- * nx / tx <= 8 blocks; it gives the cluster kernel's results bit for bit.  Results are
+ * D3Q19 lattices in FP32/FP16/BF16 with nx % 32 == 0 and ny % 8 == 0 run a TMA-staged
+ * kernel when tx x ty is 32 x 8, 32 x 4 (nx <= 256), 64 x 4 (nx % 64 == 0) or one of the
+ * 512-node tiles 32 x 16 and 64 x 8 (D3Q19 only), the generic kernel otherwise.  The CG and
+ * SC-multiphase models without walls or the repulsion force run the pair kernel (two nodes
+ * per thread, clusters of nx / 32 blocks, nx <= 512), which picks its own shape whichever of
+ * these tilings is set; the other models run the cluster kernel (nx <= 256: clusters of
+ * nx / 32 or nx / 64 blocks that exchange the x-halo in distributed shared memory; 512-node
+ * tiles run as 32 x 8).  Results are
  * bitwise independent of the shape within each kernel; the kernels agree to a few ulps of
  * the stored populations (the compiler fuses multiply-adds differently).  LBM_EINVAL for
  * shapes outside those limits. */
