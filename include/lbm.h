@@ -173,14 +173,12 @@ const char* lbm_status_string(lbm_status s);
  * ceil(nz / tz) chunks of near-equal length, one block per unit (tz must be 1 for D2Q9).
  * tz = 0: a persistent grid of as many blocks as fit on the device looping over the units,
  * with a chunk count chosen from that block count.  Default 32 x 8 x 16.
- * D3Q19 lattices in FP32/FP16/BF16 with nx % 32 == 0 and ny % 8 == 0 run a TMA-staged
- * kernel when tx x ty is 32 x 8, 32 x 4 (nx <= 256), 64 x 4 (nx % 64 == 0) or one of the
- * 512-node tiles 32 x 16 and 64 x 8 (D3Q19 only), the generic kernel otherwise.  The CG and
- * SC-multiphase models without walls or the repulsion force run the pair kernel (two nodes
- * per thread, clusters of nx / 32 blocks, nx <= 512), which picks its own shape whichever of
- * these tilings is set; the other models run the cluster kernel (nx <= 256: clusters of
- * nx / 32 or nx / 64 blocks that exchange the x-halo in distributed shared memory; 512-node
- * tiles run as 32 x 8).  Results are
+ * The tiling only applies to the generic kernel.  D3Q19 lattices in FP32/FP16/BF16 with two
+ * buffers and nx <= 512 run the pair kernel (two nodes per thread), which picks its own
+ * shape, except with the repulsion force and, when nx % 32 != 0 or ny % 8 != 0, below 300,000
+ * nodes (600,000 in 16-bit storage with walls) with walls, 16-bit storage or the SC-multiphase
+ * model; wider ones with nx % 32 == 0 and ny % 8 == 0 run a TMA-staged kernel when tx x ty is
+ * 32 x 8 (which the 512-node tiles 32 x 16 and 64 x 8 stand for).  Results are
  * bitwise independent of the shape within each kernel; the kernels agree to a few ulps of
  * the stored populations (the compiler fuses multiply-adds differently).  LBM_EINVAL for
  * shapes outside those limits. */

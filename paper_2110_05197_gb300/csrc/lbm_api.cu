@@ -92,11 +92,15 @@ size_t workspace_layout(const lbm_params& p, lbm_ctx* c) {
   };
   // in-place streaming: one population buffer and one reference field
   const bool aa = p.streaming == LBM_STREAM_AA;
-  const size_t of0 = take((size_t)K * Q * N * elt);
-  const size_t of1 = aa ? of0 : take((size_t)K * Q * N * elt);
-  const size_t or0 = take((size_t)K * N * relt);
-  const size_t or1 = aa ? or0 : take((size_t)K * N * relt);
+  const int px = row_pitch(p);
+  const long long NS = (long long)px * p.ny * p.nz;
+  const size_t of0 = take((size_t)K * Q * NS * elt);
+  const size_t of1 = aa ? of0 : take((size_t)K * Q * NS * elt);
+  const size_t or0 = take((size_t)K * NS * relt);
+  const size_t or1 = aa ? or0 : take((size_t)K * NS * relt);
   const size_t osol = take((size_t)N);
+  const size_t onear = take((size_t)N);
+  const size_t olist = take((kWallList + 1) * sizeof(unsigned));
   // staging: rho_r, rho_b, momentum/velocity (3), then psi (SC multiphase) or the two
   // multirange Psi_s in the compute type (a seventh row for FP64 storage)
   const int stage_rows = (p.model == LBM_MODEL_SC_MR && p.precision == LBM_FP64) ? 7 : 6;
@@ -111,6 +115,10 @@ size_t workspace_layout(const lbm_params& p, lbm_ctx* c) {
     c->K = K;
     c->Q = Q;
     c->N = N;
+    c->px = px;
+    c->NS = NS;
+    c->near_wall = c->ws + onear;
+    c->wall_list = reinterpret_cast<unsigned*>(c->ws + olist);
     c->elt = elt;
     c->relt = relt;
     c->aa = aa;
@@ -165,12 +173,14 @@ static EncodeFn encode_fn() {
   return fn;
 }
 
-// 4-D view (x, array, y, z) of a [arrays][z][y][x] buffer with boxes {bx, arrays, rows, 1}.
-static bool encode4(EncodeFn fn, CUtensorMap* m, CUtensorMapDataType dt, size_t elt, void* base, int nx, int ny,
-                    int nz, int arrays, long long n, int bx, int rows) {
-  const cuuint64_t dims[4] = {(cuuint64_t)nx, (cuuint64_t)arrays, (cuuint64_t)ny, (cuuint64_t)nz};
-  const cuuint64_t strides[3] = {(cuuint64_t)(n * elt), (cuuint64_t)nx * elt, (cuuint64_t)nx * ny * elt};
-  const cuuint32_t box[4] = {(cuuint32_t)bx, (cuuint32_t)arrays, (cuuint32_t)rows, 1};
+// 4-D view (x, array, y, z) of a [arrays][z][y][x] buffer whose rows are c->px elements
+// apart, with boxes {kTmaTX, arrays, rows, 1}; what a box holds beyond nx and ny reads as 0.
+static bool encode4(EncodeFn fn, CUtensorMap* m, CUtensorMapDataType dt, size_t elt, void* base, const lbm_ctx* c,
+                    int arrays, int rows) {
+  const cuuint64_t px = c->px, ny = c->p.ny;
+  const cuuint64_t dims[4] = {(cuuint64_t)c->p.nx, (cuuint64_t)arrays, ny, (cuuint64_t)c->p.nz};
+  const cuuint64_t strides[3] = {(cuuint64_t)(c->NS * elt), px * elt, px * ny * elt};
+  const cuuint32_t box[4] = {kTmaTX, (cuuint32_t)arrays, (cuuint32_t)rows, 1};
   const cuuint32_t es[4] = {1, 1, 1, 1};
   return fn(m, dt, 4, base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -178,39 +188,25 @@ static bool encode4(EncodeFn fn, CUtensorMap* m, CUtensorMapDataType dt, size_t 
 
 bool build_tma_maps(lbm_ctx* c) {
   const lbm_params& p = c->p;
-  if (p.lattice != LBM_D3Q19 || p.precision == LBM_FP64 || c->aa) return false;
-  if (p.nx % kTmaTX != 0 || p.ny % kTmaTY != 0) return false;
-  const int K = c->K, Q = c->Q;
-  if (K * Q > 256) return false;
+  if (!pair_lattice(p) && (p.lattice != LBM_D3Q19 || p.precision == LBM_FP64 || c->aa || p.nx % kTmaTX != 0 ||
+                           p.ny % kTmaTY != 0))
+    return false;
+  const int KQ = c->K * c->Q;
   EncodeFn fn = encode_fn();
   if (!fn) return false;
   const CUtensorMapDataType dt = p.precision == LBM_FP32   ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                  : p.precision == LBM_FP16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
                                                            : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+  const CUtensorMapDataType rt = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
   for (int b = 0; b < 2; b++) {
     TmaMaps& m = c->tma[b];
-    bool ok = encode4(fn, &m.pop_main_row, dt, c->elt, c->f[b], p.nx, p.ny, p.nz, K * Q, c->N, kTmaTX, 1) &&
-              encode4(fn, &m.pop_main_mid, dt, c->elt, c->f[b], p.nx, p.ny, p.nz, K * Q, c->N, kTmaTX, kTmaTY) &&
-              encode4(fn, &m.ref_main_row, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, c->relt, c->r[b], p.nx, p.ny, p.nz, K,
-                      c->N, kTmaTX, 1) &&
-              encode4(fn, &m.ref_main_mid, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, c->relt, c->r[b], p.nx, p.ny, p.nz, K,
-                      c->N, kTmaTX, kTmaTY) &&
-              encode4(fn, &m.pop_main_mid4, dt, c->elt, c->f[b], p.nx, p.ny, p.nz, K * Q, c->N, kTmaTX, 4) &&
-              encode4(fn, &m.ref_main_mid4, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, c->relt, c->r[b], p.nx, p.ny, p.nz, K,
-                      c->N, kTmaTX, 4);
-    if (ok && p.nx % 64 == 0)
-      ok = encode4(fn, &m.pop_w_row, dt, c->elt, c->f[b], p.nx, p.ny, p.nz, K * Q, c->N, 64, 1) &&
-           encode4(fn, &m.pop_w_mid4, dt, c->elt, c->f[b], p.nx, p.ny, p.nz, K * Q, c->N, 64, 4) &&
-           encode4(fn, &m.ref_w_row, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, c->relt, c->r[b], p.nx, p.ny, p.nz, K, c->N,
-                   64, 1) &&
-           encode4(fn, &m.ref_w_mid4, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, c->relt, c->r[b], p.nx, p.ny, p.nz, K, c->N,
-                   64, 4);
-    if (!ok) return false;
-    // tiles of 16 rows (lbm_step_pair.cuh); optional
-    m.mid16 = p.ny % 16 == 0 &&
-              encode4(fn, &m.pop_main_mid16, dt, c->elt, c->f[b], p.nx, p.ny, p.nz, K * Q, c->N, kTmaTX, 16) &&
-              encode4(fn, &m.ref_main_mid16, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, c->relt, c->r[b], p.nx, p.ny, p.nz, K,
-                      c->N, kTmaTX, 16);
+    if (!encode4(fn, &m.pop_main_row, dt, c->elt, c->f[b], c, KQ, 1) ||
+        !encode4(fn, &m.pop_main_mid, dt, c->elt, c->f[b], c, KQ, 8) ||
+        !encode4(fn, &m.pop_main_mid16, dt, c->elt, c->f[b], c, KQ, 16) ||
+        !encode4(fn, &m.ref_main_row, rt, c->relt, c->r[b], c, c->K, 1) ||
+        !encode4(fn, &m.ref_main_mid, rt, c->relt, c->r[b], c, c->K, 8) ||
+        !encode4(fn, &m.ref_main_mid16, rt, c->relt, c->r[b], c, c->K, 16))
+      return false;
   }
   return true;
 }
@@ -300,6 +296,7 @@ lbm_status lbm_init_fields(lbm_ctx* c, const double* rho_r, const double* rho_b,
       e = cudaMemcpyAsync(c->solid, solid, N, cudaMemcpyHostToDevice, c->stream);
     }
     c->has_walls = true;
+    if (e == cudaSuccess && lbm::pair_lattice(c->p)) e = lbm::launch_near_wall(c);
   } else {
     e = cudaMemsetAsync(c->solid, 0, N, c->stream);
     c->has_walls = false;
@@ -429,6 +426,21 @@ lbm_status lbm_destroy(lbm_ctx* c) {
 
 uint64_t lbm_launch_count(const lbm_ctx* c) { return c ? c->launches : 0; }
 
+namespace {
+// Copies `rows` rows of nx elements between a stored array (rows c->px apart) and a dense
+// buffer.
+cudaError_t copy_rows(lbm_ctx* c, void* dense, void* stored, size_t rows, size_t elt, bool to_dense) {
+  const size_t w = c->p.nx * elt, pitch = c->px * elt;
+  if (w == pitch)
+    return to_dense ? cudaMemcpyAsync(dense, stored, rows * w, cudaMemcpyDefault, c->stream)
+                    : cudaMemcpyAsync(stored, dense, rows * w, cudaMemcpyDefault, c->stream);
+  return to_dense ? cudaMemcpy2DAsync(dense, w, stored, pitch, w, rows, cudaMemcpyDefault, c->stream)
+                  : cudaMemcpy2DAsync(stored, pitch, dense, w, w, rows, cudaMemcpyDefault, c->stream);
+}
+// Rows of a whole set of `arrays` stored arrays.
+size_t all_rows(const lbm_ctx* c, int arrays) { return (size_t)arrays * c->p.ny * c->p.nz; }
+}  // namespace
+
 size_t lbm_state_bytes(const lbm_ctx* c) {
   if (!c) return 0;
   return (size_t)c->K * c->Q * c->N * c->elt + (size_t)c->K * c->N * c->relt;
@@ -457,11 +469,9 @@ lbm_status lbm_save_state(lbm_ctx* c, void* dst) {
                               c->stream);
       }
   } else {
-    e = cudaMemcpyAsync(dst, c->f[b], fb, cudaMemcpyDefault, c->stream);
+    e = copy_rows(c, dst, c->f[b], all_rows(c, c->K * c->Q), c->elt, true);
   }
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(static_cast<char*>(dst) + fb, c->r[b], (size_t)c->K * c->N * c->relt, cudaMemcpyDefault,
-                        c->stream);
+  if (e == cudaSuccess) e = copy_rows(c, static_cast<char*>(dst) + fb, c->r[b], all_rows(c, c->K), c->relt, true);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return fail(c, e);
   return hd.status ? LBM_EUNSTABLE : LBM_OK;
@@ -480,24 +490,17 @@ lbm_status copy_planes(lbm_ctx* c, int32_t z0, int32_t np, void* buf, bool to_bu
   if (!c || !buf || z0 < 0 || np < 1 || z0 + np > c->p.nz) return LBM_EINVAL;
   if (c->sticky != LBM_OK) return c->sticky;
   if (!c->initialised || c->aa) return LBM_ESTATE;
-  const size_t plane = (size_t)c->p.nx * c->p.ny;
-  const size_t pb = np * plane * c->elt, rb = np * plane * c->relt;
+  const size_t rows = (size_t)np * c->p.ny, first = (size_t)z0 * c->p.ny * c->px;
+  const size_t pb = rows * c->p.nx * c->elt, rb = rows * c->p.nx * c->relt;
   unsigned char* f = static_cast<unsigned char*>(c->f[c->cur]);
   unsigned char* r = static_cast<unsigned char*>(c->r[c->cur]);
   unsigned char* b = static_cast<unsigned char*>(buf);
   cudaError_t e = cudaSuccess;
-  for (int a = 0; a < c->K * c->Q && e == cudaSuccess; a++) {
-    unsigned char* st = f + ((size_t)a * c->N + z0 * plane) * c->elt;
-    unsigned char* bb = b + a * pb;
-    e = to_buf ? cudaMemcpyAsync(bb, st, pb, cudaMemcpyDefault, c->stream)
-               : cudaMemcpyAsync(st, bb, pb, cudaMemcpyDefault, c->stream);
-  }
-  for (int k = 0; k < c->K && e == cudaSuccess; k++) {
-    unsigned char* st = r + ((size_t)k * c->N + z0 * plane) * c->relt;
-    unsigned char* bb = b + (size_t)c->K * c->Q * pb + k * rb;
-    e = to_buf ? cudaMemcpyAsync(bb, st, rb, cudaMemcpyDefault, c->stream)
-               : cudaMemcpyAsync(st, bb, rb, cudaMemcpyDefault, c->stream);
-  }
+  for (int a = 0; a < c->K * c->Q && e == cudaSuccess; a++)
+    e = copy_rows(c, b + a * pb, f + ((size_t)a * c->NS + first) * c->elt, rows, c->elt, to_buf);
+  for (int k = 0; k < c->K && e == cudaSuccess; k++)
+    e = copy_rows(c, b + (size_t)c->K * c->Q * pb + k * rb, r + ((size_t)k * c->NS + first) * c->relt, rows, c->relt,
+                  to_buf);
   return e == cudaSuccess ? LBM_OK : fail(c, e);
 }
 }  // namespace
@@ -518,16 +521,17 @@ lbm_status lbm_load_state(lbm_ctx* c, const void* src, const uint8_t* solid) {
   if (solid) {
     e = cudaMemcpyAsync(c->solid, solid, N, cudaMemcpyDefault, c->stream);
     c->has_walls = true;
+    if (e == cudaSuccess && lbm::pair_lattice(c->p)) e = lbm::launch_near_wall(c);
   } else {
     e = cudaMemsetAsync(c->solid, 0, N, c->stream);
     c->has_walls = false;
   }
   const size_t fb = (size_t)c->K * c->Q * N * c->elt;
-  const size_t rb = (size_t)c->K * N * c->relt;
+  void* dense = const_cast<void*>(src);
   for (int b = 0; b < (c->aa ? 1 : 2) && e == cudaSuccess; b++) {
-    e = cudaMemcpyAsync(c->f[b], src, fb, cudaMemcpyDefault, c->stream);
+    e = copy_rows(c, dense, c->f[b], all_rows(c, c->K * c->Q), c->elt, false);
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(c->r[b], static_cast<const char*>(src) + fb, rb, cudaMemcpyDefault, c->stream);
+      e = copy_rows(c, static_cast<char*>(dense) + fb, c->r[b], all_rows(c, c->K), c->relt, false);
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(c->diag, 0, sizeof(lbm_diag), c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);

@@ -50,6 +50,8 @@ struct AuxParams {
   double body[3];
   double umax, neg_tol;
   double Ga[2], Gr[2];   // multirange SC self-couplings
+  int px;                // row pitch and size of the stored arrays
+  long long ns;
   int aa;                // in-place streaming: the state's layout parity is its buffer index
 };
 
@@ -60,6 +62,8 @@ AuxParams aux_params(const lbm_ctx* c) {
   a.ny = q.ny;
   a.nz = q.nz;
   a.n = c->N;
+  a.px = c->px;
+  a.ns = c->NS;
   a.aa = c->aa;
   a.model = q.model;
   a.enhanced = q.enhanced_eq;
@@ -171,16 +175,17 @@ __global__ void init_eq_kernel(S* __restrict__ fa, S* __restrict__ fb, RT* __res
                                const double* __restrict__ U, const uint8_t* __restrict__ solid,
                                const step_t<S>* __restrict__ fc, AuxParams a) {
   using C = step_t<S>;
-  const I N = I(a.n);
+  const I N = I(a.n), NS = I(a.ns);
   for (I n = blockIdx.x * I(blockDim.x) + threadIdx.x; n < N; n += I(gridDim.x) * blockDim.x) {
     C out[L::Q];
+    const I st = stored_index(n, a.nx, a.px);
     if (solid && solid[n]) {
       for (int k = 0; k < a.K; k++) {
-        ra[I(k) * N + n] = RT(0);
-        if (rb_) rb_[I(k) * N + n] = RT(0);
+        ra[I(k) * NS + st] = RT(0);
+        if (rb_) rb_[I(k) * NS + st] = RT(0);
         for (int i = 0; i < L::Q; i++) {
-          fa[I(k * L::Q + i) * N + n] = from_d<S>(0.0);
-          if (fb) fb[I(k * L::Q + i) * N + n] = from_d<S>(0.0);
+          fa[I(k * L::Q + i) * NS + st] = from_d<S>(0.0);
+          if (fb) fb[I(k * L::Q + i) * NS + st] = from_d<S>(0.0);
         }
       }
       continue;
@@ -211,9 +216,9 @@ __global__ void init_eq_kernel(S* __restrict__ fa, S* __restrict__ fb, RT* __res
           grad_c<L, C>(phi, solid, n, x, y, z, a, g);
       }
       feq_dev<L, C>(C(phi[n]), a.phi[k], en, u, g, C(phi[n] - (double)rref), out);
-      ra[I(k) * N + n] = rref;
+      ra[I(k) * NS + st] = rref;
       for (int i = 0; i < L::Q; i++) {
-        fa[I(k * L::Q + i) * N + n] = st_s<S, C>(out[i]);
+        fa[I(k * L::Q + i) * NS + st] = st_s<S, C>(out[i]);
       }
     }
   }
@@ -228,16 +233,17 @@ template <class S, class RT>
 __global__ void restore_plane_kernel(S* __restrict__ fa, S* __restrict__ fb, RT* __restrict__ ra,
                                      RT* __restrict__ rb_, const double* __restrict__ plane,
                                      const double* __restrict__ acc, const uint8_t* __restrict__ solid, long long n,
-                                     long long off, long long roff, double phi, bool write_ref) {
+                                     long long off, long long roff, double phi, bool write_ref, int nx, int px) {
   for (long long m = blockIdx.x * (long long)blockDim.x + threadIdx.x; m < n; m += (long long)gridDim.x * blockDim.x) {
     const bool wall = solid && solid[m];
     const RT r = wall ? RT(0) : RT(acc[m]);
     const S v = wall ? from_d<S>(0.0) : from_d<S>(plane[m] - phi * (double)r);
-    fa[off + m] = v;
-    if (fb) fb[off + m] = v;
+    const long long st = stored_index(m, nx, px);
+    fa[off + st] = v;
+    if (fb) fb[off + st] = v;
     if (write_ref) {
-      ra[roff + m] = r;
-      if (rb_) rb_[roff + m] = r;
+      ra[roff + st] = r;
+      if (rb_) rb_[roff + st] = r;
     }
   }
 }
@@ -257,9 +263,11 @@ __global__ void export_kernel(const S* __restrict__ f0, const S* __restrict__ f1
     const int plane = first_plane + (int)(m / a.n);
     const long long node = m - (long long)(plane - first_plane) * a.n;
     const int k = plane / L::Q, i = plane - k * L::Q;
-    out[m] = (solid && solid[node]) ? 0.0
-                                    : to_d(f[aa_index_n<L>(k, i, node, a.nx, a.ny, a.nz, a.n, odd)]) +
-                                          a.phi[k][grp<L>(i)] * to_d(r[(long long)k * a.n + node]);
+    const long long st = stored_index(node, a.nx, a.px);
+    out[m] = (solid && solid[node])
+                 ? 0.0
+                 : to_d(f[odd ? aa_index_n<L>(k, i, node, a.nx, a.ny, a.nz, a.n, odd) : (k * L::Q + i) * a.ns + st]) +
+                       a.phi[k][grp<L>(i)] * to_d(r[k * a.ns + st]);
   }
 }
 
@@ -288,25 +296,29 @@ __global__ void densities_kernel(const S* __restrict__ f0, const S* __restrict__
   const S* f = b ? f1 : f0;
   const RT* r = b ? r1 : r0;
   const bool odd = a.aa && (b & 1);
-  const I N = I(a.n);
+  const I N = I(a.n), NS = I(a.ns);
   for (I m = blockIdx.x * I(blockDim.x) + threadIdx.x; m < N; m += I(gridDim.x) * blockDim.x) {
     // momentum summed exactly (ExactSum): the colours' momenta nearly cancel at
     // interfaces, so rounding in the sum would show up in the reported u; the shift
     // phi_i r is symmetric in c_i and carries no momentum: opposite pairs of the stored
     // deviations
     ExactSum<C> jx, jy, jz;
+    const I st = stored_index(m, a.nx, a.px);
+    auto at = [&](int k, int i) -> I {
+      return odd ? aa_index_nt<L, I>(k, i, m, a.nx, a.ny, a.nz, N, odd) : I(k * L::Q + i) * NS + st;
+    };
     for (int k = 0; k < 2; k++) {
       double s = 0.0;
       if (k < a.K) {
-        ExactSum<C> acc{static_cast<C>(r[I(k) * N + m])};  // sum_i phi_i = 1
+        ExactSum<C> acc{static_cast<C>(r[I(k) * NS + st])};  // sum_i phi_i = 1
 #pragma unroll
         for (int i = 0; i < L::Q; i++)
-          acc.add(ld_s<S, C>(f[aa_index_nt<L, I>(k, i, m, a.nx, a.ny, a.nz, N, odd)]));
+          acc.add(ld_s<S, C>(f[at(k, i)]));
         s = acc.value();
 #pragma unroll
         for (int q = 0; q < L::NP; q++) {
-          const C vp = ld_s<S, C>(f[aa_index_nt<L, I>(k, 2 * q + 1, m, a.nx, a.ny, a.nz, N, odd)]);
-          const C vm = ld_s<S, C>(f[aa_index_nt<L, I>(k, 2 * q + 2, m, a.nx, a.ny, a.nz, N, odd)]);
+          const C vp = ld_s<S, C>(f[at(k, 2 * q + 1)]);
+          const C vm = ld_s<S, C>(f[at(k, 2 * q + 2)]);
           if (L::pcx(q)) { jx.add(L::pcx(q) > 0 ? vp : -vp); jx.add(L::pcx(q) > 0 ? -vm : vm); }
           if (L::pcy(q)) { jy.add(L::pcy(q) > 0 ? vp : -vp); jy.add(L::pcy(q) > 0 ? -vm : vm); }
           if (L::pcz(q)) { jz.add(L::pcz(q) > 0 ? vp : -vp); jz.add(L::pcz(q) > 0 ? -vm : vm); }
@@ -549,6 +561,25 @@ __global__ void __launch_bounds__(kDiagThreads) diag_kernel(const double* __rest
 }
 
 
+// Which nodes are walls or have one beside them, and a list of the latter
+// (lbm_step_pair.cuh).
+__global__ void near_wall_kernel(const uint8_t* __restrict__ solid, uint8_t* __restrict__ near,
+                                 unsigned* __restrict__ list, AuxParams a) {
+  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < a.n; n += (long long)gridDim.x * blockDim.x) {
+    int x, y, z;
+    node_xyz(n, a, x, y, z);
+    bool beside = false;
+#pragma unroll
+    for (int i = 1; i < D3Q19::Q; i++)
+      beside |= solid[nb_index_t<long long>(x, y, z, cx<D3Q19>(i), cy<D3Q19>(i), cz<D3Q19>(i), a.nx, a.ny, a.nz)] != 0;
+    near[n] = (solid[n] ? kWallSelf : 0) | (beside ? kWallNear : 0);
+    if (beside && !solid[n]) {
+      const unsigned at = atomicAdd(&list[0], 1u);
+      if (at < kWallList) list[1 + at] = (unsigned)n;
+    }
+  }
+}
+
 int grid_for(long long n, int threads, int cap) {
   long long b = (n + threads - 1) / threads;
   if (b > cap) b = cap;
@@ -574,7 +605,7 @@ cudaError_t init_t(lbm_ctx* c, const double* rr, const double* rb, const double*
   }
   // in-place streaming: one buffer pair (the second pointers alias the first)
   // 32-bit indices where every index (populations K Q N, velocity 3 N) fits
-  auto kern = (long long)c->K * c->Q * c->N < (1LL << 31) ? init_eq_kernel<L, S, RT, int>
+  auto kern = (long long)c->K * c->Q * c->NS < (1LL << 31) ? init_eq_kernel<L, S, RT, int>
                                                           : init_eq_kernel<L, S, RT, long long>;
   kern<<<grid_for(c->N, 256, 8192), 256, 0, c->stream>>>(
       static_cast<S*>(c->f[0]), c->aa ? nullptr : static_cast<S*>(c->f[1]), static_cast<RT*>(c->r[0]),
@@ -589,8 +620,8 @@ cudaError_t restore_t(lbm_ctx* c, const double* plane, int k, int i, const doubl
   restore_plane_kernel<S, RT><<<grid_for(c->N, 256, 8192), 256, 0, c->stream>>>(
       static_cast<S*>(c->f[0]), c->aa ? nullptr : static_cast<S*>(c->f[1]), static_cast<RT*>(c->r[0]),
       c->aa ? nullptr : static_cast<RT*>(c->r[1]),
-      plane, acc + (long long)k * c->N, c->has_walls ? c->solid : nullptr, c->N, (long long)(k * c->Q + i) * c->N,
-      (long long)k * c->N, phi[k][grp<L>(i)], i == 0);
+      plane, acc + (long long)k * c->N, c->has_walls ? c->solid : nullptr, c->N, (long long)(k * c->Q + i) * c->NS,
+      (long long)k * c->NS, phi[k][grp<L>(i)], i == 0, c->p.nx, c->px);
   return cudaGetLastError();
 }
 
@@ -623,7 +654,7 @@ cudaError_t diag_t(lbm_ctx* c, double* uo) {
   double* jm = c->stage + 2 * c->N;   // momentum, then (if requested here) the velocity
   double* psi = c->stage + 5 * c->N;  // SC multiphase psi (FP64), or the multirange Psi_s
   step_t<S>* mrpsi = c->p.model == LBM_MODEL_SC_MR ? reinterpret_cast<step_t<S>*>(psi) : nullptr;
-  auto dens = (long long)c->K * c->Q * c->N < (1LL << 31) ? densities_kernel<L, S, RT, int>
+  auto dens = (long long)c->K * c->Q * c->NS < (1LL << 31) ? densities_kernel<L, S, RT, int>
                                                           : densities_kernel<L, S, RT, long long>;
   dens<<<grid_for(c->N, 256, 8192), 256, 0, c->stream>>>(f0, f1, r0, r1, c->diag, c->cur, rr, rb, psi, jm, mrpsi, a);
   cudaError_t e = cudaGetLastError();
@@ -686,6 +717,14 @@ struct DiagOp {
 cudaError_t launch_init_eq(lbm_ctx* c, const double* rr, const double* rb, const double* u) {
   c->launches += 1;
   return by_lattice_precision<InitOp>(c, rr, rb, u);
+}
+
+cudaError_t launch_near_wall(lbm_ctx* c) {
+  cudaError_t e = cudaMemsetAsync(c->wall_list, 0, sizeof(unsigned), c->stream);
+  if (e != cudaSuccess) return e;
+  c->launches += 1;
+  near_wall_kernel<<<grid_for(c->N, 256, 8192), 256, 0, c->stream>>>(c->solid, c->near_wall, c->wall_list, aux_params(c));
+  return cudaGetLastError();
 }
 
 cudaError_t launch_restore_accumulate(lbm_ctx* c, const double* plane, int k, double* acc, bool first) {

@@ -8,6 +8,7 @@
 
 #include "../../include/lbm.h"
 #include "lbm_step.cuh"
+#include "lbm_step_pair.cuh"
 #include "lbm_step_tma.cuh"
 
 // Device-side diagnostics record: totals (LBM_NTOTALS doubles) then the blow-up status.
@@ -25,17 +26,21 @@ struct lbm_ctx {
   lbm_params p;
   int K, Q;
   long long N;
+  int px;                // nodes from one row of a stored array to the next (row_pitch)
+  long long NS;          // elements of a stored array: px * ny * nz
   size_t elt;            // bytes per stored population
   size_t relt;           // bytes per reference density
   cudaStream_t stream;
   unsigned char* ws;
   size_t ws_bytes;
-  void* f[2];            // A/B population buffers [K][Q][N], deviations from phi * r
-  void* r[2];            // A/B reference densities [K][N] (paired with f[])
+  void* f[2];            // A/B population buffers [K][Q][NS], deviations from phi * r
+  void* r[2];            // A/B reference densities [K][NS] (paired with f[])
   int cur;               // index of the buffer pair holding the current state
   bool aa;               // in-place streaming: f[1] == f[0], r[1] == r[0], and cur is the
                          // layout parity of the state (lbm_step_aa.cuh)
   uint8_t* solid;        // [N] wall mask (all zero without walls)
+  uint8_t* near_wall;    // [N] kWallSelf for a wall, kWallNear beside one (pair kernel)
+  unsigned* wall_list;   // the nodes beside a wall (kWallList)
   bool has_walls;
   double* stage;         // [6][N] FP64 staging ([7][N] for the multirange model in FP64):
                          // rho_r, rho_b, momentum then u (x, y, z), psi (SC multiphase) or
@@ -55,7 +60,7 @@ struct lbm_ctx {
   bool rep;              // CG repulsion force enabled (rep_pi != 0)
   void* colour;          // [N] rho^N (step compute type), repulsion pre-pass
   void* normals;         // [3][N] unit colour gradients, repulsion pre-pass
-  bool tma_ok;           // tensor maps built: the TMA-staged kernel can run this lattice
+  bool tma_ok;           // tensor maps built: the TMA-staged kernels can run this lattice
   lbm::TmaMaps tma[2];   // maps for reading buffer pair 0 / 1
 };
 
@@ -79,14 +84,27 @@ cudaError_t launch_step_f32(lbm_ctx* c);
 cudaError_t launch_step_f16(lbm_ctx* c);
 cudaError_t launch_step_bf16(lbm_ctx* c);
 size_t step_smem_for(const lbm_ctx* c, int tx, int ty);
-// Encode the tensor maps of both buffer pairs when the lattice suits the TMA-staged
-// kernel (D3Q19, FP32/FP16/BF16 storage, nx % 32 == 0, ny % 8 == 0); false otherwise.
+// Encode the tensor maps of both buffer pairs when the lattice suits a TMA-staged kernel:
+// pair_lattice, or D3Q19 in FP32/FP16/BF16 with nx % 32 == 0 and ny % 8 == 0; false otherwise.
 bool build_tma_maps(lbm_ctx* c);
+
+// Whether a lattice is stored for the pair kernel (lbm_step_pair.cuh): D3Q19, 32- or 16-bit
+// storage, two buffers, at most kPairMaxCluster tiles of 32 columns.  (The repulsion force
+// runs elsewhere, on the same storage.)
+inline bool pair_lattice(const lbm_params& p) {
+  return p.lattice == LBM_D3Q19 && p.precision != LBM_FP64 && p.streaming == LBM_STREAM_AB &&
+         p.model != LBM_MODEL_SC_MR && p.nx <= 32 * kPairMaxCluster;
+}
+// Row pitch of the stored arrays: a tensor map needs rows of a multiple of 16 bytes, i.e. 8
+// elements of the narrowest storage; other lattices are stored densely.
+inline int row_pitch(const lbm_params& p) { return pair_lattice(p) ? (p.nx + 7) / 8 * 8 : p.nx; }
 
 // Aux launchers (lbm_aux.cu)
 cudaError_t launch_init_eq(lbm_ctx* c, const double* rr, const double* rb, const double* u);
 // Checkpoint restore in two passes over the populations: accumulate the densities
 // (acc [K][N] FP64), then write deviations relative to them.
+// near_wall and wall_list of the current wall mask.
+cudaError_t launch_near_wall(lbm_ctx* c);
 cudaError_t launch_restore_accumulate(lbm_ctx* c, const double* plane, int k, double* acc, bool first);
 cudaError_t launch_restore_plane(lbm_ctx* c, const double* plane, int k, int i, const double* acc);
 cudaError_t launch_export_plane(lbm_ctx* c, double* plane, int k, int i);
@@ -130,6 +148,8 @@ StepParams<T> make_step_params(const lbm_ctx* c) {
   s.nchunks = c->tz > 0 ? (q.nz + c->tz - 1) / c->tz : 1;
   s.nblk = s.ncol * s.nchunks;
   s.n = c->N;
+  s.px = c->px;
+  s.ns = c->NS;
   double phi[2][3];
   rest_weights(q, phi);
   for (int k = 0; k < 2; k++)

@@ -82,4 +82,15 @@ __device__ __forceinline__ void node_coords(long long n, int nx, int ny, long lo
   }
 }
 
+// Index in a stored array, whose rows are px nodes apart, of node n (its own index where the
+// rows are dense).
+template <class I>
+__device__ __forceinline__ I stored_index(I n, int nx, int px) {
+  if (px == nx) return n;
+  if constexpr (sizeof(I) == 4)
+    return n + I(unsigned(n) / unsigned(nx)) * (px - nx);
+  else
+    return n + n / nx * (px - nx);
+}
+
 }  // namespace lbm

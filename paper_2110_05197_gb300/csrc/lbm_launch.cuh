@@ -7,7 +7,6 @@
 #include "lbm_internal.cuh"
 #include "lbm_step_aa.cuh"
 #include "lbm_step_pair.cuh"
-#include "lbm_step_tmac.cuh"
 
 namespace lbm {
 
@@ -15,14 +14,16 @@ namespace lbm {
 // is in the odd in-place layout
 template <class L, class T, class S, class RT>
 __global__ void colour_kernel(const S* __restrict__ f, const RT* __restrict__ r, T* __restrict__ colour,
-                              RepParams a, int odd) {
+                              RepParams a, int odd, int px, long long ns) {
   for (long long m = blockIdx.x * (long long)blockDim.x + threadIdx.x; m < a.n; m += (long long)gridDim.x * blockDim.x) {
     T rho[2];
+    const long long st = stored_index(m, a.nx, px);
     for (int k = 0; k < 2; k++) {
       T g[L::Q];
 #pragma unroll
-      for (int i = 0; i < L::Q; i++) g[i] = ld_s<S, T>(f[aa_index_n<L>(k, i, m, a.nx, a.ny, a.nz, a.n, odd)]);
-      rho[k] = comp_state<L, T, RT>(g, T(r[(long long)k * a.n + m])).rho;
+      for (int i = 0; i < L::Q; i++)
+        g[i] = ld_s<S, T>(f[odd ? aa_index_n<L>(k, i, m, a.nx, a.ny, a.nz, a.n, odd) : (k * L::Q + i) * ns + st]);
+      rho[k] = comp_state<L, T, RT>(g, T(r[k * ns + st])).rho;
     }
     T s0 = rho[0], s1 = rho[1];
     if (a.color_norm) {
@@ -57,7 +58,8 @@ cudaError_t launch_rep_prepass_t(lbm_ctx* c, int buf) {
   const int grid = (int)std::min<long long>((c->N + 255) / 256, 8192);
   colour_kernel<L, T, S, RT><<<grid, 256, 0, c->stream>>>(static_cast<const S*>(c->f[buf]),
                                                            static_cast<const RT*>(c->r[buf]),
-                                                           static_cast<T*>(c->colour), a, c->aa ? (buf & 1) : 0);
+                                                           static_cast<T*>(c->colour), a, c->aa ? (buf & 1) : 0,
+                                                           c->px, c->NS);
   if (3 * c->N < (1LL << 31))  // 32-bit indices: the normals array holds 3 N values
     normals_kernel<L, T, int><<<grid, 256, 0, c->stream>>>(
         static_cast<const T*>(c->colour), c->has_walls ? c->solid : nullptr, static_cast<T*>(c->normals), a);
@@ -116,60 +118,12 @@ cudaError_t launch_tma_t(lbm_ctx* c) {
   return cudaGetLastError();
 }
 
-// TMA-staged kernel with the x-halo exchanged inside a cluster of nx / 32 blocks.
-template <class L, class T, class S, class RT, int MODEL, bool WALLS, int TX, int TY>
-cudaError_t launch_tmac_t(lbm_ctx* c) {
-  constexpr size_t smem = tmac_smem_bytes<L, T, S, RT, MODEL, WALLS, TX, TY>();
-  auto kern = step_kernel_tmac<L, T, S, RT, MODEL, WALLS, TX, TY>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
-  const int C = c->p.nx / TX;
-  StepParams<T> sp = make_step_params<T>(c);
-  sp.ncx = C;                // blocks per cluster
-  sp.ncol = c->p.ny / TY;    // tile rows: the work partition's columns
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = C;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(tmac_threads<MODEL, S, TX, TY>(), 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = c->stream;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (c->tz > 0) {
-    sp.nblk = sp.ncol * sp.nchunks;
-  } else {
-    const void* fn = reinterpret_cast<const void*>(kern);
-    if (c->occ_fn != fn || c->occ_tx != -C) {
-      int ncl = 0;
-      cfg.gridDim = dim3(C, 1, 1);
-      cudaError_t e = cudaOccupancyMaxActiveClusters(&ncl, kern, &cfg);
-      if (e != cudaSuccess) return e;
-      c->occ_fn = fn;
-      c->occ_tx = -C;
-      c->occ_ty = 0;
-      c->occ_blocks = ncl > 0 ? ncl : 1;
-    }
-    persistent_plan(sp, c->occ_blocks);  // clusters
-  }
-  cfg.gridDim = dim3(sp.nblk * C, 1, 1);
-  S* fout = static_cast<S*>(c->f[c->cur ^ 1]);
-  RT* rout = static_cast<RT*>(c->r[c->cur ^ 1]);
-  return cudaLaunchKernelEx(&cfg, kern, c->tma[c->cur], fout, rout, c->solid, &c->diag->status, sp);
-}
-
 // Pair kernel (lbm_step_pair.cuh): clusters of nx / 32 blocks, each cluster one run of
 // (tile row, plane) pairs; TY rows per tile, MB blocks per SM.
-template <class L, class T, class S, class RT, int MODEL, int TY, int MB>
+template <class L, class T, class S, class RT, int MODEL, int FORM, int TY, int MB>
 cudaError_t launch_pair_tile(lbm_ctx* c) {
   constexpr size_t smem = pair_smem_bytes<L, S, RT, MODEL, TY>(pair_raw<L, S, RT, MODEL, TY, MB>());
-  auto kern = step_kernel_pair<L, T, S, RT, MODEL, TY, MB>;
+  auto kern = step_kernel_pair<L, T, S, RT, MODEL, FORM, TY, MB>;
   static bool attr_set = false;
   if (!attr_set) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -177,10 +131,10 @@ cudaError_t launch_pair_tile(lbm_ctx* c) {
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  const int C = c->p.nx / kPairTX;
+  const int C = (c->p.nx + kPairTX - 1) / kPairTX;
   StepParams<T> sp = make_step_params<T>(c);
-  sp.ncx = C;               // blocks per cluster
-  sp.ncol = c->p.ny / TY;   // tile rows
+  sp.ncx = C;                         // blocks per cluster
+  sp.ncol = (c->p.ny + TY - 1) / TY;  // tile rows
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = C;
@@ -206,37 +160,51 @@ cudaError_t launch_pair_tile(lbm_ctx* c) {
   sp.nblk = (int)std::min<long long>(c->occ_blocks, (long long)sp.ncol * sp.nz);  // clusters
   cfg.gridDim = dim3(sp.nblk * C, 1, 1);
   OutArrays<S, RT, ModelTraits<MODEL>::K * L::Q, ModelTraits<MODEL>::K> out;
-  for (int a = 0; a < c->K * c->Q; a++) out.f[a] = static_cast<S*>(c->f[c->cur ^ 1]) + a * c->N;
-  for (int k = 0; k < c->K; k++) out.r[k] = static_cast<RT*>(c->r[c->cur ^ 1]) + k * c->N;
-  return cudaLaunchKernelEx(&cfg, kern, c->tma[c->cur], out, &c->diag->status, sp);
+  for (int a = 0; a < c->K * c->Q; a++) out.f[a] = static_cast<S*>(c->f[c->cur ^ 1]) + a * c->NS;
+  for (int k = 0; k < c->K; k++) out.r[k] = static_cast<RT*>(c->r[c->cur ^ 1]) + k * c->NS;
+  return cudaLaunchKernelEx(&cfg, kern, c->tma[c->cur], out, static_cast<const uint8_t*>(c->near_wall),
+                            &c->diag->status, sp);
 }
 
-// Tile of the pair kernel.  CG keeps a plane's sums in registers: 242 of them, two blocks of
-// 4 warps per SM.  SC in FP32 runs 16 warps per SM as two blocks of 16 rows, whose halo rows
-// cost 12% of the staging instead of 25% with 8 rows (128^3: 68 us against 73), unless there
-// are fewer tiles of 16 rows than blocks to hold them (32^3: 10.4 us against 8.8); in 16-bit
-// storage, whose plane buffers are half as large, as four blocks of 8 rows (57.6 against
-// 59.8 us).
-template <class L, class T, class S, class RT, int MODEL>
+// Tile of the pair kernel.  CG keeps a plane's sums in registers (242 of them), two-component
+// SC two sets: two blocks of 4 warps per SM.  SC multiphase in FP32 runs 16 warps per SM as
+// two blocks of 16 rows, whose halo rows cost 12% of the staging instead of 25% with 8 rows
+// (128^3: 68 us against 73), unless 16 rows do not divide ny or there are fewer such tiles
+// than blocks to hold them (32^3: 10.4 us against 8.8); in 16-bit storage, whose plane
+// buffers are half as large, as four blocks of 8 rows (57.6 against 59.8 us).
+template <class L, class T, class S, class RT, int MODEL, bool WALLS>
 cudaError_t launch_pair_t(lbm_ctx* c) {
-  if constexpr (MODEL == kCG) {
-    return launch_pair_tile<L, T, S, RT, MODEL, 8, 2>(c);
-  } else if constexpr (sizeof(S) == 4) {
-    const bool many = c->N / (32 * 16) >= 2 * c->nsm;
-    if (c->tma[0].mid16 && c->tma[1].mid16 && many) return launch_pair_tile<L, T, S, RT, MODEL, 16, 2>(c);
-    return launch_pair_tile<L, T, S, RT, MODEL, 8, 3>(c);
+  constexpr int MB = MODEL != kSCMP ? 2 : sizeof(S) == 4 ? 3 : 4;
+  if constexpr (WALLS) {
+    cudaError_t e = launch_pair_tile<L, T, S, RT, MODEL, kWalls, 8, MB>(c);
+    if (e != cudaSuccess) return e;
+    c->launches += 1;
+    const int grid = (int)std::min<long long>((c->N + 63) / 64, 8LL * c->nsm);
+    wall_step_kernel<L, T, S, RT, MODEL><<<grid, 64, 0, c->stream>>>(
+        static_cast<const S*>(c->f[c->cur]), static_cast<S*>(c->f[c->cur ^ 1]), static_cast<const RT*>(c->r[c->cur]),
+        static_cast<const RT*>(c->r[c->cur ^ 1]), c->solid, c->near_wall, c->wall_list, &c->diag->status,
+        make_step_params<T>(c));
+    return cudaGetLastError();
   } else {
-    return launch_pair_tile<L, T, S, RT, MODEL, 8, 4>(c);
+    if (c->p.nx % kPairTX != 0 || c->p.ny % 8 != 0) return launch_pair_tile<L, T, S, RT, MODEL, kRagged, 8, MB>(c);
+    if constexpr (MODEL == kSCMP && sizeof(S) == 4)
+      if (c->p.ny % 16 == 0 && c->N / (32 * 16) >= 2 * c->nsm)
+        return launch_pair_tile<L, T, S, RT, MODEL, kFull, 16, 2>(c);
+    return launch_pair_tile<L, T, S, RT, MODEL, kFull, 8, MB>(c);
   }
 }
 
-// Whether the pair kernel runs a lattice (of a model it has, without walls or the repulsion
-// force) at this context's tiling: every tiling that names a TMA-staged kernel.
-inline bool pair_runs(const lbm_ctx* c) {
-  if (!c->tma_ok || c->aa || c->p.nx / kPairTX > kPairMaxCluster || c->N >= (1LL << 31)) return false;
-  const int tx = c->tx, ty = c->ty;
-  if (tx == 64 && (ty == 4 || ty == 8)) return c->p.nx % 64 == 0 || ty == 8;
-  return tx == 32 && (ty == 8 || ty == 16 || (ty == 4 && c->p.nx <= 256));
+// Whether the pair kernel steps a lattice.  On aligned ones it is the fastest.  With partial
+// tiles, tuned generic tiles are as fast or faster for the cheap planes of small lattices
+// (61 x 57 x 59: SC FP32 16.6 against 20.7 us, CG FP16 27.0 against 28.9; 75 x 77 x 71: SC FP32
+// 30.9 against 26.8, CG FP16 55.7 against 47.9) and with walls, which cost a second launch
+// (75 x 77 x 71: CG FP32 74.7 against 65.8, FP16 63.8 against 62.0, SC FP16 33.5 against 39.1);
+// FP32 CG and two-component SC without walls gain or are level at every size.
+inline bool pair_steps(const lbm_ctx* c) {
+  if (!c->tma_ok || !pair_lattice(c->p)) return false;
+  const bool aligned = c->p.nx % kPairTX == 0 && c->p.ny % 8 == 0;
+  const bool cheap = c->p.model == LBM_MODEL_SC_MP || c->elt == 2 || c->has_walls;
+  return aligned || !cheap || c->N >= (c->has_walls && c->elt == 2 ? 600000 : 300000);
 }
 
 // Field-pass step (in-place streaming, or the multirange model): the field pass, then the
@@ -348,10 +316,11 @@ cudaError_t launch_step_t(lbm_ctx* c) {
     return launch_fp_t<L, T, S, RT, MODEL, WALLS, REP>(c);
   } else {
   if (c->aa) return launch_fp_t<L, T, S, RT, MODEL, WALLS, REP>(c);
-  if constexpr (L::D == 3 && sizeof(T) == 4 && !WALLS && !REP && (MODEL == kCG || MODEL == kSCMP))
-    if (pair_runs(c)) return launch_pair_t<L, T, S, RT, MODEL>(c);
+  // the pair kernel, whatever the tiling
+  if constexpr (L::D == 3 && sizeof(T) == 4 && !REP)
+    if (pair_steps(c)) return launch_pair_t<L, T, S, RT, MODEL, WALLS>(c);
   if (c->tx * c->ty > 256) {
-    // a 512-node tiling the pair kernel does not take: the 32 x 8 persistent tiling
+    // the 512-node tilings run as 32 x 8 persistent tiles
     const int tx = c->tx, ty = c->ty, tz = c->tz;
     c->tx = kTmaTX;
     c->ty = kTmaTY;
@@ -362,18 +331,10 @@ cudaError_t launch_step_t(lbm_ctx* c) {
     c->tz = tz;
     return e;
   }
-  if constexpr (L::D == 3 && sizeof(T) == 4 && !REP) {
-   if constexpr (WALLS || MODEL == kSC2C) {
-    const bool small_index = (long long)c->K * c->Q * c->N < (1LL << 31);
-    if (c->tma_ok && c->tx == 64 && c->ty == 4 && c->p.nx % 64 == 0 && c->p.nx / 64 <= kMaxCluster && small_index)
-      return launch_tmac_t<L, T, S, RT, MODEL, WALLS, 64, 4>(c);
-    if (c->tma_ok && c->tx == kTmaTX && c->ty == 4 && c->p.nx / kTmaTX <= kMaxCluster && small_index)
-      return launch_tmac_t<L, T, S, RT, MODEL, WALLS, kTmaTX, 4>(c);
-    if (c->tma_ok && c->tx == kTmaTX && c->ty == kTmaTY && c->p.nx / kTmaTX <= kMaxCluster && small_index)
-      return launch_tmac_t<L, T, S, RT, MODEL, WALLS, kTmaTX, kTmaTY>(c);
-   }
-    if (c->tma_ok && c->tx == kTmaTX && c->ty == kTmaTY) return launch_tma_t<L, T, S, RT, MODEL, WALLS>(c);
-  }
+  if constexpr (L::D == 3 && sizeof(T) == 4 && !REP)
+    if (c->tma_ok && c->px == c->p.nx && c->p.nx % kTmaTX == 0 && c->p.ny % kTmaTY == 0 && c->tx == kTmaTX &&
+        c->ty == kTmaTY)
+      return launch_tma_t<L, T, S, RT, MODEL, WALLS>(c);
   if constexpr (REP) {
     cudaError_t e = launch_rep_prepass_t<L, T, S, RT>(c, c->cur);
     if (e != cudaSuccess) return e;
@@ -381,7 +342,7 @@ cudaError_t launch_step_t(lbm_ctx* c) {
   // 32-bit node and array indices where every index fits (FP64 storage keeps 64-bit ones:
   // its step is bound by the FP64 rate, not by index arithmetic)
   if constexpr (sizeof(T) < 8) {
-    if ((long long)c->K * c->Q * c->N < (1LL << 31)) return launch_generic_t<L, T, S, RT, MODEL, WALLS, REP, int>(c);
+    if ((long long)c->K * c->Q * c->NS < (1LL << 31)) return launch_generic_t<L, T, S, RT, MODEL, WALLS, REP, int>(c);
   }
   return launch_generic_t<L, T, S, RT, MODEL, WALLS, REP, long long>(c);
   }

@@ -52,6 +52,8 @@ struct StepParams {
   int nchunks;            // z-chunks per column
   int nblk;               // blocks in the grid (WorkRange)
   long long n;            // nodes
+  int px;                 // nodes from one stored row to the next
+  long long ns;           // elements of a stored array (px * ny * nz)
   T phi[2][3];            // rest-state weights per component and group (CG: Eq. phi; SC: w)
   // CG
   T inv_nu_r, inv_nu_b;   // 1/nu_k, nu_k = (tau_k - 1/2)/3
@@ -561,7 +563,7 @@ struct StepArrays {
 // a block barrier, so the caller may reuse shared memory right away.
 // REP (CG only): add the repulsion force of Eq. repForce from the pre-pass fields
 // colour / normals (lbm_rep.cuh).  I: the integer type of node and array indices, int
-// when K * Q * N < 2^31 (the launcher's choice), else long long.
+// when K * Q * ns < 2^31 (the launcher's choice), else long long.
 template <class L, class T, class S, class RT, int MODEL, bool WALLS, bool REP, class I = long long>
 __device__ __forceinline__ void march_segment(const StepArrays<S, RT>& a, const StepParams<T>& p,
                                               const T* __restrict__ colour, const T* __restrict__ normals,
@@ -581,7 +583,7 @@ __device__ __forceinline__ void march_segment(const StepArrays<S, RT>& a, const 
   const int EX = TX + 2;
   const int NE = EX * (TY + 2), NI = TX * TY;
   const int tid = threadIdx.y * TX + threadIdx.x;
-  const I N = I(p.n);
+  const I N = I(p.ns);
   const int x0 = (sg.col % p.ncx) * TX, y0 = (sg.col / p.ncx) * TY;
 
   T* fld = reinterpret_cast<T*>(smem_raw);           // [NPL][NV][NE]
@@ -596,7 +598,7 @@ __device__ __forceinline__ void march_segment(const StepArrays<S, RT>& a, const 
     for (int e = tid; e < NE; e += NI) {
       const int ey = e / EX, ex = e - ey * EX;
       const int gx = wrap(x0 - 1 + ex, p.nx), gy = wrap(y0 - 1 + ey, p.ny);
-      const I n = gx + I(p.nx) * (gy + I(p.ny) * gz);
+      const I row = gy + I(p.ny) * gz, n = gx + I(p.px) * row;
       const bool inner = pb >= 0 && ex >= 1 && ex <= TX && ey >= 1 && ey <= TY;
       const int ii = (ey - 1) * TX + (ex - 1);
       T rho[2] = {T(0), T(0)};
@@ -619,7 +621,7 @@ __device__ __forceinline__ void march_segment(const StepArrays<S, RT>& a, const 
       node_fields<MODEL, T>(p, rho[0], rho[1], out);
 #pragma unroll
       for (int f = 0; f < NF; f++) fld[(sl * NV + f) * NE + e] = out[f];
-      if (WALLS) msk[sl * NE + e] = solid[n];
+      if (WALLS) msk[sl * NE + e] = solid[gx + I(p.nx) * row];
     }
   };
 
@@ -659,7 +661,7 @@ __device__ __forceinline__ void march_segment(const StepArrays<S, RT>& a, const 
     }
     // new reference densities of this node
     const int zz = z, zm = zz == 0 ? p.nz - 1 : zz - 1, zpp = zz + 1 >= p.nz ? 0 : zz + 1;
-    const I n0 = gx + I(p.nx) * (gy + I(p.ny) * zz);
+    const I n0 = gx + I(p.px) * (gy + I(p.ny) * zz);
 #pragma unroll
     for (int k = 0; k < K; k++) rout[I(k) * N + n0] = RT(cs[k].q);
     // push to y = x + c_i (periodic), re-referenced to phi_i q(y); halfway bounce-back to
@@ -670,7 +672,7 @@ __device__ __forceinline__ void march_segment(const StepArrays<S, RT>& a, const 
       const int X = dxv == 0 ? gx : (dxv > 0 ? xp : xm);
       const int Y = dyv == 0 ? gy : (dyv > 0 ? yp : ym);
       const int Z = dzv == 0 ? zz : (dzv > 0 ? zpp : zm);
-      I nd = X + I(p.nx) * (Y + I(p.ny) * Z);
+      I nd = X + I(p.px) * (Y + I(p.ny) * Z);
       int id = i;
       const int sl = slot_of(dzv);
       const int ed = e0 + dyv * EX + dxv;

@@ -1,6 +1,6 @@
 // D3Q19 step kernel on pairs of nodes: every thread owns two nodes, neighbours along y, of a
-// 32 x TY tile and marches z (FP32 and 16-bit storage; colour-gradient and Shan-Chen
-// multiphase models).
+// 32 x TY tile and marches z (FP32 and 16-bit storage; the colour-gradient, Shan-Chen
+// multiphase and two-component models; any nx up to 512, any ny and nz, walls).
 //
 // Same step and densities as the other step kernels (lbm_step.cuh); what differs is the
 // work per instruction.  The step is bound by issued instructions rather than bytes (a
@@ -22,7 +22,7 @@
 //      cluster spans a full x-row of tiles, so the periodic wrap in x stays inside it) as
 //      asynchronous remote stores that complete on the receiver's mbarrier of slot J;
 //   3. collides its nodes of plane J-1 from the sums t_i it kept (CG: both colours'
-//      deviations added, since the CG collision acts on the total; SC: the deviations) and
+//      deviations added, since the CG collision acts on the total; SC: the deviations of each component) and
 //      the field slots J-2, J-1, J, and pushes the results.  The wait for the neighbours'
 //      columns of plane J comes after the part of the collision that does not read them
 //      (moments, relaxation rate, in-plane differences): at 128^3 (clusters of 4) 152 ->
@@ -42,7 +42,7 @@
 // slots.  Every wait is bounded (lbm_step_tma.cuh).
 #pragma once
 
-#include "lbm_step_tmac.cuh"
+#include "lbm_step_tma.cuh"
 #include "lbm_vec.cuh"
 
 namespace lbm {
@@ -176,12 +176,18 @@ __device__ __forceinline__ void cg_collide_pair(const StepParams<float>& p, cons
   const F2 inv_g = each(gabs, [&](float a) { return a > eps ? rcp_newton(a) : 0.f; });
   const F2 Ag = each(gabs, [&](float a) { return a > eps ? p.A * a : 0.f; });
   const F2 cR = qR * inv;
-  const F2 rec = F2(p.beta) * cR * (qB * inv);
+  const F2 qRB = cR * qB;
+  const F2 rec = F2(p.beta) * qRB * inv;
   const F2 wrho = omega * rho;
   const F2 kg = fma(F2(-0.5f), omega, F2(1.f));
   const F2 uF = fma(u[0], F[0], fma(u[1], F[1], u[2] * F[2]));
   F2 K0[3], K1[3], K2[3], K3[3], K4[3], base[3], rcg[3], S0[3], S1[3];
   const F2 pe = Ag * inv_g * inv_g;
+  // 3 w_i and 3/2 w_i in FP32 with the sums over the directions that conserve momentum (3 w_1
+  // * 2 + 3 w_2 * 8 = 1) and mass (to 3/2) exactly.  Rounded to nearest, 3 w_i gains 3e-8 of
+  // the momentum every step, the same way at every node.
+  const float w3[3] = {1.f, 11184810.f / 67108864.f, 11184811.f / 134217728.f};
+  const float w32[3] = {16777215.f / 33554432.f, 11184811.f / 134217728.f, 11184811.f / 268435456.f};
 #pragma unroll
   for (int g = 0; g <= 2; g++) {
     const float wg = float(L::w(g)), phR = p.phi[0][g], phB = p.phi[1][g];
@@ -189,20 +195,26 @@ __device__ __forceinline__ void cg_collide_pair(const StepParams<float>& p, cons
     const F2 kgs = fma(F2(phR), cr.d, F2(phB) * cb.d);
     F2 e = fma(F2(phR), cr.dq, F2(phB) * cb.dq);
     e = fma(F2(float(L::psi(g))) * en, ugr, e);
-    e = fma(F2(-1.5f * wg) * rho, uu, e);
+    e = fma(F2(-w32[g]) * rho, uu, e);
     K0[g] = fma(om1, kgs, fma(omega, e, F2(float(-L::B(g))) * Ag));
     if (forced) K0[g] = fma(F2(-3.f * wg) * kg, uF, K0[g]);
-    base[g] = (qR * F2(phB) * qB - qB * F2(phR) * qR) * inv;
     if (g > 0) {
       K1[g] = F2(4.5f * wg) * wrho;
       K2[g] = F2(float(2.0 * L::xi(g))) * (omega * en);
       K3[g] = F2(wg) * pe;
-      K4[g] = F2(3.f * wg) * wrho;
+      K4[g] = F2(w3[g]) * wrho;
       rcg[g] = rec * fma(qR, F2(phR), qB * F2(phB)) * inv_g * F2(g == 1 ? 1.f : 0.70710678118654752440f);
       S0[g] = F2(9.f * wg) * kg;
-      S1[g] = F2(3.f * wg) * kg;
+      S1[g] = F2(w3[g]) * kg;
     }
   }
+  // (rho_R phi^B q_B - rho_B phi^R q_R) / rho with q = rho.  The rest direction takes what
+  // makes the sum over the directions vanish: the rounded constants' own sum is off by up to
+  // 3e-8, the same way at every node and step, and would move that much of one colour to the
+  // other (velocity error after 40 steps 1.9e-6, against 8e-7).
+  base[1] = qRB * F2(p.phi[1][1] - p.phi[0][1]);
+  base[2] = qRB * F2(p.phi[1][2] - p.phi[0][2]);
+  base[0] = fma(F2(-12.f), base[2], F2(-6.f) * base[1]);
   {
     const F2 Gs = fma(om1, t[0], K0[0]);
     const F2 gR = fma(cR, Gs, base[0]);
@@ -297,6 +309,76 @@ __device__ __forceinline__ void scmp_collide_pair(const StepParams<float>& p, co
   }
 }
 
+// Two-component SC collision (Eqs. doublebeltrepulsionforce2, guoforce2, collisSC, equiliSC,
+// source) of a thread's two nodes; t[0..Q) and t[Q..2Q): the components' deviations; nb(f,
+// i, j): field f = q_1, q_2; per component as in scmp_collide_pair, with the common velocity.
+template <class L, class NB, class READY, class EMIT>
+__device__ __forceinline__ void sc2c_collide_pair(const StepParams<float>& p, const F2 (&t)[2 * L::Q],
+                                                  const Comp2 (&c)[2], const NB& nb, const READY& ready,
+                                                  const EMIT& emit) {
+  constexpr int Q = L::Q;
+  PairSum<L> s1, s2, sj;
+#pragma unroll
+  for (int q = 0; q < L::NP; q++)
+    sj.add(q, (t[2 * q + 1] - t[2 * q + 2]) + (t[Q + 2 * q + 1] - t[Q + 2 * q + 2]));
+  auto diffs = [&](bool inplane) {
+#pragma unroll
+    for (int q = 0; q < L::NP; q++) {
+      if ((L::pcz(q) == 0) != inplane) continue;
+      F2 d1, d2;
+#pragma unroll
+      for (int j = 0; j < 2; j++) {
+        d1.set(j, nb(0, 2 * q + 1, j) - nb(0, 2 * q + 2, j));
+        d2.set(j, nb(1, 2 * q + 1, j) - nb(1, 2 * q + 2, j));
+      }
+      s1.add(q, d1);
+      s2.add(q, d2);
+    }
+  };
+  diffs(true);
+  ready();
+  diffs(false);
+  const F2 inv = each(c[0].q + c[1].q, [](float a) { return rcp_newton(a); });
+  F2 u[3], F[2][3];
+#pragma unroll
+  for (int k = 0; k < 3; k++) {
+    const F2 w1 = F2(float(L::w(1))), w2 = F2(float(L::w(2)));
+    F[0][k] = F2(-p.G) * c[0].q * fma(w2, s2.dg[k], w1 * s2.ax[k]);
+    F[1][k] = F2(-p.G) * c[1].q * fma(w2, s1.dg[k], w1 * s1.ax[k]);
+    if (p.has_body) {
+      const F2 b = F2(p.body[k]) * inv;
+      F[0][k] = fma(b, c[0].q, F[0][k]);
+      F[1][k] = fma(b, c[1].q, F[1][k]);
+    }
+    u[k] = fma(F2(0.5f), F[0][k] + F[1][k], sj.ax[k] + sj.dg[k]) * inv;
+  }
+  const F2 uu = fma(u[0], u[0], fma(u[1], u[1], u[2] * u[2]));
+#pragma unroll
+  for (int s = 0; s < 2; s++) {
+    const float omega = s == 0 ? p.omega_r : p.omega_b, kg = 1.f - 0.5f * omega;
+    const F2 om1 = F2(1.f - omega), wr = F2(omega) * c[s].q;
+    const F2 uF = fma(u[0], F[s][0], fma(u[1], F[s][1], u[2] * F[s][2]));
+    F2 av[3], bv[3];
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+      av[k] = fma(F2(3.f) * wr, u[k], F2(3.f * kg) * F[s][k]);
+      bv[k] = fma(F2(4.5f) * wr, u[k], F2(9.f * kg) * F[s][k]);
+    }
+    F2 K0 = fma(om1, c[s].d, F2(omega) * c[s].dq);
+    K0 = fma(F2(-1.5f) * wr, uu, K0);
+    K0 = fma(F2(-3.f * kg), uF, K0);
+    emit(s, 0, fma(om1, t[s * Q], F2(float(L::w(0))) * K0));
+#pragma unroll
+    for (int q = 0; q < L::NP; q++) {
+      const F2 wg = F2(float(L::w(L::pgrp(q))));
+      const F2 cu = dot2<L>(q, u), ca = dot2<L>(q, av), cb = dot2<L>(q, bv);
+      const F2 E = fma(cu, cb, K0);
+      emit(s, 2 * q + 1, fma(wg, E + ca, om1 * t[s * Q + 2 * q + 1]));
+      emit(s, 2 * q + 2, fma(wg, E - ca, om1 * t[s * Q + 2 * q + 2]));
+    }
+  }
+}
+
 template <int MODEL>
 struct PairTraits;
 template <>
@@ -304,11 +386,19 @@ struct PairTraits<kCG> {
   // q_R, q_B, rho^N, and their sum rho: the gradient reads rho 18 times per node, which as
   // q_R + q_B would take two loads and an addition each
   static constexpr int NV = 4;
+  static constexpr int NH = 1;  // held values per direction: the colours' sum
   static constexpr bool EARLY = true;
 };
 template <>
 struct PairTraits<kSCMP> {
   static constexpr int NV = 2;  // psi, q
+  static constexpr int NH = 1;
+  static constexpr bool EARLY = false;
+};
+template <>
+struct PairTraits<kSC2C> {
+  static constexpr int NV = 2;  // q_1, q_2
+  static constexpr int NH = 2;
   static constexpr bool EARLY = false;
 };
 
@@ -345,6 +435,23 @@ struct PlaneRun {
   }
 };
 
+__device__ __forceinline__ uint32_t cluster_ctarank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// shared::cluster address of the same shared-memory offset in block `rank` of the cluster
+__device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
+  uint32_t d;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(addr), "r"(rank));
+  return d;
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile(
+      "barrier.cluster.arrive.release.aligned;\n\t"
+      "barrier.cluster.wait.acquire.aligned;" ::
+          : "memory");
+}
 // Asynchronous 32-bit store into another block's shared memory (addresses from mapa);
 // completion is counted, in bytes, on that block's mbarrier `bar`.
 __device__ __forceinline__ void st_async_f32(uint32_t cluster_addr, float v, uint32_t cluster_bar) {
@@ -381,14 +488,27 @@ struct OutArrays {
   RT* r[K];
 };
 
-// Launch: cluster dims (C, 1, 1) with C = p.ncx = nx / 32 <= kPairMaxCluster; grid = p.nblk
-// clusters * C blocks of 16 TY threads, MB blocks per SM; p.ncol = ny / TY tile rows.
-// Every index within an array fits 31 bits.
-template <class L, class T, class S, class RT, int MODEL, int TY, int MB>
+constexpr uint8_t kWallSelf = 1, kWallNear = 2;  // near_wall: a wall node; a neighbour is a wall
+// wall_list: their number, then the nodes beside a wall in any order, if there are at most
+// kWallList of them.
+constexpr unsigned kWallList = 1u << 17;
+
+// Forms of the kernel: every tile full (nx % 32 == 0, ny % TY == 0); any size; any size with
+// walls.  The tests for partial tiles cost the full ones 4% (CG 128^3 FP32) to 16% (FP16).
+enum PairForm : int { kFull = 0, kRagged = 1, kWalls = 2 };
+
+// Launch: cluster dims (C, 1, 1) with C = p.ncx = ceil(nx / 32) <= kPairMaxCluster; grid =
+// p.nblk clusters * C blocks of 16 TY threads, MB blocks per SM; p.ncol = ceil(ny / TY) tile
+// rows.  Rows are p.px nodes apart (a multiple of 16 bytes, which a tensor map needs), the
+// last tile of a row or column may be partial.  Every index within an array fits 31 bits.
+// With walls (kWalls) the nodes beside one are left to wall_step_kernel, except for their
+// reference densities, which it reads.
+template <class L, class T, class S, class RT, int MODEL, int FORM, int TY, int MB>
 __global__ void __launch_bounds__(16 * TY, MB)
     step_kernel_pair(const __grid_constant__ TmaMaps maps,
                      const __grid_constant__ OutArrays<S, RT, ModelTraits<MODEL>::K * L::Q, ModelTraits<MODEL>::K> out,
-                     int* __restrict__ status, const __grid_constant__ StepParams<T> p) {
+                     const uint8_t* __restrict__ near_wall, int* __restrict__ status,
+                     const __grid_constant__ StepParams<T> p) {
   static_assert(sizeof(T) == 4 && sizeof(RT) == 4, "fields are exchanged as 32-bit words");
   static_assert(TY == 8 || TY == 16, "tile rows with a tensor map");
   constexpr int TX = kPairTX, kWarps = TY / 2;
@@ -397,11 +517,9 @@ __global__ void __launch_bounds__(16 * TY, MB)
   static_assert(EARLY || RAW >= 2, "late sums keep a plane's buffer through the next copy");
   using Lay = TmaLayout<L, S, RT, MODEL, TX, TY>;
   constexpr int Q = L::Q, K = Lay::K;
-  constexpr int NV = PairTraits<MODEL>::NV;
+  constexpr int NV = PairTraits<MODEL>::NV, NH = PairTraits<MODEL>::NH;
   constexpr int EX = Lay::EX, NE = Lay::NE;
   constexpr int FS = kPairFields;
-  // bytes of the two halo columns (all TY + 2 rows, NV fields) the x-neighbours send
-  constexpr uint32_t kEdgeBytes = 2u * (TY + 2) * NV * 4u;
   // A blown-up (or timed-out) state stops stepping; the cluster barriers are still passed.
   const bool skip = *status != 0;
 
@@ -416,8 +534,11 @@ __global__ void __launch_bounds__(16 * TY, MB)
   const uint32_t rank = cluster_ctarank();
   const uint32_t left = (rank + C - 1) % C, right = (rank + 1) % C;
   const int x0 = (int)rank * TX;
+  constexpr bool FULL = FORM == kFull, WALLS = FORM == kWalls;
+  const int width = FULL ? TX : min(TX, p.nx - x0);                                // columns of this tile
+  const int left_width = FULL || rank != 0 ? TX : p.nx - (C - 1) * TX;  // and of the left neighbour's
   const int cid = blockIdx.x / C;
-  const int plane_n = p.nx * p.ny;
+  const int plane_n = p.px * p.ny;
 
   if (tid == 0) {
     for (int s = 0; s < RAW; s++) mbar_init(&raw_full[s], 1);
@@ -440,7 +561,7 @@ __global__ void __launch_bounds__(16 * TY, MB)
   // TMA copy of one plane into raw buffer s: top halo row, TY rows, bottom halo row
   auto issue = [&](const PlaneRun& pr, int s) {
     const int y0 = pr.sg.col * TY;
-    const int yt = y0 == 0 ? p.ny - 1 : y0 - 1, yb = y0 + TY == p.ny ? 0 : y0 + TY;
+    const int yt = y0 == 0 ? p.ny - 1 : y0 - 1, yb = y0 + TY >= p.ny ? 0 : y0 + TY;
     const int gz = wrap(pr.z, p.nz);
     unsigned char* b = bufs + s * Lay::BUF_MAIN;
     uint64_t* bar = &raw_full[s];
@@ -470,9 +591,10 @@ __global__ void __launch_bounds__(16 * TY, MB)
   for (int j = 0; j < (EARLY ? RAW : RAW - 1); j++) issue_next();
 
   // state of the plane staged last, collided one plane later
-  F2 hold[Q], next_hold[Q];
+  F2 hold[NH * Q], next_hold[EARLY ? Q : 1];
   Comp2 hcs[K];
   int prev_z = 0, prev_y0 = 0;
+  int near[2] = {0, 0};
   bool prev_interior = false;
 
   for (int J = 0; cur.valid; J++) {
@@ -482,13 +604,26 @@ __global__ void __launch_bounds__(16 * TY, MB)
     const int fs = J % FS;
     const unsigned char* b = bufs + (J % RAW) * Lay::BUF_MAIN;
     const int halo_warp = J % kWarps;  // stages the halo rows too
+    const int rows = FULL ? TY : min(TY, p.ny - y0);
     Comp2 cs[K];
+    // what the nodes of plane J are: outside the lattice (as kWallSelf), a wall, beside one
+    int next_near[2] = {0, 0};
+    if constexpr (!FULL) {
+#pragma unroll
+      for (int j = 0; j < 2; j++) {
+        const int gy = y0 + 2 * warp + j;
+        next_near[j] = lane >= width || gy >= p.ny ? kWallSelf : 0;
+        if (WALLS && interior && next_near[j] == 0) next_near[j] = near_wall[x0 + lane + p.nx * (gy + p.ny * z)];
+      }
+    }
     // ---- stage plane J ----
     if (alive) wait(&raw_full[J % RAW], J / RAW);
-    if (alive && tid == 0) mbar_arrive_expect_tx(&fld_full[fs], kEdgeBytes);
+    // bytes of the two halo columns (rows + 2 rows, NV fields) the x-neighbours send
+    if (alive && tid == 0) mbar_arrive_expect_tx(&fld_full[fs], 2u * (rows + 2) * NV * 4u);
     if (alive) {
-      // densities and fields of the extended rows ey0, ey1; the sums too when `own`
-      auto stage_rows = [&](int ey0, int ey1, bool own, Comp2 (&c)[K]) {
+      // densities and fields of the raw rows ey0, ey1, into field rows fy0, fy1 (negative:
+      // none); the sums too when `own`
+      auto stage_rows = [&](int ey0, int ey1, int fy0, int fy1, bool own, Comp2 (&c)[K]) {
         const S* p0 = reinterpret_cast<const S*>(b + Lay::PM::row(ey0)) + lane;
         const S* p1 = reinterpret_cast<const S*>(b + Lay::PM::row(ey1)) + lane;
         const RT* r0 = reinterpret_cast<const RT*>(b + Lay::OFF_RM + Lay::RMR::row(ey0)) + lane;
@@ -512,7 +647,8 @@ __global__ void __launch_bounds__(16 * TY, MB)
         float* f = fld + fs * NV * NE + lane + 1;
 #pragma unroll
         for (int j = 0; j < 2; j++) {
-          const int e = (j == 0 ? ey0 : ey1) * EX;
+          const int fy = j == 0 ? fy0 : fy1, e = fy * EX;
+          if (!FULL && (fy < 0 || lane >= width)) continue;
           float fields[2];
           node_fields<MODEL, float>(p, c[0].q[j], K == 2 ? c[K - 1].q[j] : 0.f, fields);
           if constexpr (MODEL == kCG) {
@@ -520,44 +656,57 @@ __global__ void __launch_bounds__(16 * TY, MB)
             f[NE + e] = c[1].q[j];
             f[2 * NE + e] = fields[1];
             f[3 * NE + e] = fields[0];
+          } else if constexpr (MODEL == kSC2C) {
+            f[e] = c[0].q[j];
+            f[NE + e] = c[1].q[j];
           } else {
             f[e] = fields[0];
             f[NE + e] = c[0].q[j];
           }
         }
       };
-      stage_rows(2 * warp + 1, 2 * warp + 2, true, cs);
+      if (FULL || 2 * warp < rows)
+        stage_rows(2 * warp + 1, 2 * warp + 2, 2 * warp + 1, FULL || 2 * warp + 1 < rows ? 2 * warp + 2 : -1, true, cs);
       if (warp == halo_warp) {
         Comp2 unused[K];
-        stage_rows(0, TY + 1, false, unused);
+        stage_rows(0, TY + 1, 0, rows + 1, false, unused);
       }
     }
     __syncthreads();  // local fields of plane J complete; iteration J-1 retired
     issue_next();     // into this plane's buffer (EARLY), else into plane J-1's
-    if (alive && (lane == 0 || lane == TX - 1)) {
+    if (alive && (lane == 0 || lane == width - 1)) {
       // the tile's first column is the left neighbour's right halo column, its last
       // column the right neighbour's left one
-      const uint32_t peer = lane == 0 ? left : right;
-      const int exd = lane == 0 ? TX + 1 : 0;
-      const uint32_t bar = mapa_shared(smem_addr(&fld_full[fs]), peer);
-      auto send = [&](int ey) {  // the fields this thread staged in row ey
+      auto send_column = [&](uint32_t peer, int exd) {
+        const uint32_t bar = mapa_shared(smem_addr(&fld_full[fs]), peer);
+        auto send = [&](int ey) {  // the fields this thread staged in row ey
 #pragma unroll
-        for (int f = 0; f < NV; f++) {
-          const float* src = &fld[(fs * NV + f) * NE + ey * EX];
-          st_async_f32(mapa_shared(smem_addr(src + exd), peer), src[lane + 1], bar);
+          for (int f = 0; f < NV; f++) {
+            const float* src = &fld[(fs * NV + f) * NE + ey * EX];
+            st_async_f32(mapa_shared(smem_addr(src + exd), peer), src[lane + 1], bar);
+          }
+        };
+        if (FULL || 2 * warp < rows) send(2 * warp + 1);
+        if (FULL || 2 * warp + 1 < rows) send(2 * warp + 2);
+        if (warp == halo_warp) {
+          send(0);
+          send(rows + 1);
         }
       };
-      send(2 * warp + 1);
-      send(2 * warp + 2);
-      if (warp == halo_warp) {
-        send(0);
-        send(TY + 1);
+      if constexpr (FULL) {
+        send_column(lane == 0 ? left : right, lane == 0 ? TX + 1 : 0);
+      } else {
+        if (lane == 0) send_column(left, left_width + 1);
+        if (lane == width - 1) send_column(right, 0);
       }
     }
     auto ready = [&]() { wait(&fld_full[fs], J / FS); };  // the neighbours' columns of plane J
     if (alive && !prev_interior) ready();
     // ---- collide plane J-1 ----
-    if (alive && prev_interior) {
+    const bool any_live = FULL || __any_sync(0xffffffffu, near[0] == 0 || near[1] == 0 || near[0] == kWallNear ||
+                                                              near[1] == kWallNear);
+    if (alive && prev_interior && !any_live) ready();  // walls, or rows beyond a partial tile
+    if (alive && prev_interior && any_live) {
       const int slm = (J + FS - 2) % FS, sl0 = (J + FS - 1) % FS;
       const int e0 = (2 * warp + 1) * EX + (lane + 1);
       const float* f_m = fld + slm * NV * NE + e0;
@@ -567,11 +716,11 @@ __global__ void __launch_bounds__(16 * TY, MB)
         const float* base = cz<L>(i) == 0 ? f_0 : (cz<L>(i) > 0 ? f_p : f_m);
         return base[f * NE + (cy<L>(i) + j) * EX + cx<L>(i)];
       };
-      // node indices: columns x-1 .. x+1, rows y-1 .. y+2, planes z-1 .. z+1 (periodic)
+      // storage indices: columns x-1 .. x+1, rows y-1 .. y+2, planes z-1 .. z+1 (periodic)
       const int gx = x0 + lane, gy = prev_y0 + 2 * warp, zz = prev_z;
+      auto row = [&](int y) { return unsigned((y >= p.ny ? y - p.ny : y) * p.px); };
       const unsigned xo[3] = {unsigned(gx == 0 ? p.nx - 1 : gx - 1), unsigned(gx), unsigned(gx + 1 >= p.nx ? 0 : gx + 1)};
-      const unsigned yo[4] = {unsigned((gy == 0 ? p.ny - 1 : gy - 1) * p.nx), unsigned(gy * p.nx),
-                              unsigned((gy + 1) * p.nx), unsigned((gy + 2 >= p.ny ? 0 : gy + 2) * p.nx)};
+      const unsigned yo[4] = {row(gy == 0 ? p.ny - 1 : gy - 1), row(gy), row(gy + 1), row(gy + 2)};
       const unsigned zo[3] = {unsigned((zz == 0 ? p.nz - 1 : zz - 1) * plane_n), unsigned(zz * plane_n),
                               unsigned((zz + 1 >= p.nz ? 0 : zz + 1) * plane_n)};
       auto dest = [&](int i, int j) -> unsigned {
@@ -580,7 +729,8 @@ __global__ void __launch_bounds__(16 * TY, MB)
 #pragma unroll
       for (int k = 0; k < K; k++)
 #pragma unroll
-        for (int j = 0; j < 2; j++) out.r[k][dest(0, j)] = hcs[k].q[j];
+        for (int j = 0; j < 2; j++)
+          if (FULL || !(near[j] & kWallSelf)) out.r[k][dest(0, j)] = hcs[k].q[j];
       // a result of component k, re-referenced to the destination's density (field f), out
       auto push = [&](int k, int f, int i, const F2& v) {
         F2 o = v;
@@ -591,7 +741,8 @@ __global__ void __launch_bounds__(16 * TY, MB)
           o = fma(F2(p.phi[k][grp<L>(i)]), hcs[k].q - n, v);
         }
 #pragma unroll
-        for (int j = 0; j < 2; j++) out.f[k * Q + i][dest(i, j)] = st_s<S, T>(o[j]);
+        for (int j = 0; j < 2; j++)
+          if (FULL || near[j] == 0) out.f[k * Q + i][dest(i, j)] = st_s<S, T>(o[j]);
       };
       if constexpr (MODEL == kCG) {
         auto emit = [&](int i, const F2& vR, const F2& vB) {
@@ -599,6 +750,9 @@ __global__ void __launch_bounds__(16 * TY, MB)
           push(1, 1, i, vB);
         };
         cg_collide_pair<L>(p, hold, hcs[0], hcs[1], nb, ready, emit);
+      } else if constexpr (MODEL == kSC2C) {
+        auto emit = [&](int k, int i, const F2& v) { push(k, k, i, v); };
+        sc2c_collide_pair<L>(p, hold, hcs, nb, ready, emit);
       } else {
         F2 psic;
 #pragma unroll
@@ -616,13 +770,15 @@ __global__ void __launch_bounds__(16 * TY, MB)
       const S* p0 = reinterpret_cast<const S*>(b + Lay::PM::row(2 * warp + 1)) + lane;
       const S* p1 = reinterpret_cast<const S*>(b + Lay::PM::row(2 * warp + 2)) + lane;
 #pragma unroll
-      for (int i = 0; i < Q; i++) {
+      for (int i = 0; i < NH * Q; i++) {
         hold[i].set(0, ld_s<S, T>(p0[i * TX]));
         hold[i].set(1, ld_s<S, T>(p1[i * TX]));
       }
     }
 #pragma unroll
     for (int k = 0; k < K; k++) hcs[k] = cs[k];
+    near[0] = next_near[0];
+    near[1] = next_near[1];
     prev_interior = interior;
     prev_z = z;
     prev_y0 = y0;
@@ -633,6 +789,76 @@ __global__ void __launch_bounds__(16 * TY, MB)
     for (int j = max(0, issued - RAW); j < issued; j++) mbar_wait_bounded(&raw_full[j % RAW], (j / RAW) & 1);
   __syncwarp();
   cluster_sync_all();  // no block leaves while a neighbour may still write to it
+}
+
+// The nodes beside a wall, one thread per node, after the pair kernel: the same
+// step with the stencil values of a wall neighbour replaced by the centre's and halfway
+// bounce-back.  The fields are formed from the densities q the pair kernel has written.
+// (Inside the pair kernel the tests for walls of one warp in a tile held up the whole
+// cluster: CG 128 x 72 x 64 between two planes 70 us, 47 without walls.)  The list spares
+// most blocks, of which 255 registers a thread let few run at a time, a look at near_wall:
+// 20 us for the nodes of a 101 x 75 x 67 channel without it.
+template <class L, class T, class S, class RT, int MODEL>
+__global__ void __launch_bounds__(64) wall_step_kernel(
+    const S* __restrict__ fin, S* __restrict__ fout, const RT* __restrict__ rin, const RT* __restrict__ rout,
+    const uint8_t* __restrict__ solid, const uint8_t* __restrict__ near_wall, const unsigned* __restrict__ wall_list,
+    const int* __restrict__ status, const __grid_constant__ StepParams<T> p) {
+  if (*status != 0) return;
+  constexpr int Q = L::Q, K = ModelTraits<MODEL>::K, NF = ModelTraits<MODEL>::NF;
+  const size_t NS = (size_t)p.ns;
+  const unsigned listed = wall_list[0];
+  const bool scan = listed > kWallList;
+  const unsigned count = scan ? (unsigned)p.n : listed;
+  for (unsigned m = blockIdx.x * blockDim.x + threadIdx.x; m < count; m += gridDim.x * blockDim.x) {
+    const int n = scan ? (int)m : (int)wall_list[1 + m];
+    if (scan && near_wall[n] != kWallNear) continue;
+    int x, y, z;
+    node_coords(n, p.nx, p.ny, p.n, x, y, z);
+    const int X[3] = {x == 0 ? p.nx - 1 : x - 1, x, x + 1 >= p.nx ? 0 : x + 1};
+    const int Y[3] = {y == 0 ? p.ny - 1 : y - 1, y, y + 1 >= p.ny ? 0 : y + 1};
+    const int Z[3] = {z == 0 ? p.nz - 1 : z - 1, z, z + 1 >= p.nz ? 0 : z + 1};
+    unsigned to[Q];  // stored index of neighbour i
+    unsigned walls = 0;
+    T fld[NF][Q], q[K][Q], g[K][Q];
+    CompState<T> cs[K];
+#pragma unroll
+    for (int i = 0; i < Q; i++) {
+      const int row = Y[cy<L>(i) + 1] + p.ny * Z[cz<L>(i) + 1];
+      to[i] = X[cx<L>(i) + 1] + p.px * row;
+      walls |= (solid[X[cx<L>(i) + 1] + p.nx * row] ? 1u : 0u) << i;
+#pragma unroll
+      for (int k = 0; k < K; k++) q[k][i] = rout[k * NS + to[i]];
+      T out[2];
+      node_fields<MODEL, T>(p, q[0][i], q[K - 1][i], out);
+#pragma unroll
+      for (int f = 0; f < NF; f++) fld[f][i] = out[f];
+    }
+#pragma unroll
+    for (int k = 0; k < K; k++) {
+#pragma unroll
+      for (int i = 0; i < Q; i++) g[k][i] = ld_s<S, T>(fin[(k * Q + i) * NS + to[0]]);
+      cs[k] = comp_state<L, T, RT>(g[k], rin[k * NS + to[0]]);
+    }
+    auto nbr = [&](int f, int i) -> T { return (walls >> i) & 1u ? fld[f][0] : fld[f][i]; };
+    if constexpr (MODEL == kCG) {
+      const T Fx[3] = {T(0), T(0), T(0)};
+      cg_collide<L, T>(p, g, cs[0], cs[1], nbr, Fx);
+    } else if constexpr (MODEL == kSCMP) {
+      scmp_collide<L, T>(p, g, cs[0], nbr);
+    } else {
+      sc2c_collide<L, T>(p, g, cs[0], cs[1], nbr);
+    }
+#pragma unroll
+    for (int i = 0; i < Q; i++) {
+      const bool bounce = (walls >> i) & 1u;
+#pragma unroll
+      for (int k = 0; k < K; k++) {
+        T v = g[k][i];
+        if (i != 0 && !bounce) v += p.phi[k][grp<L>(i)] * (cs[k].q - q[k][i]);
+        fout[(k * Q + (bounce ? opp<L>(i) : i)) * NS + (bounce ? to[0] : to[i])] = st_s<S, T>(v);
+      }
+    }
+  }
 }
 
 }  // namespace lbm

@@ -24,14 +24,11 @@
 
 namespace lbm {
 
-// Tensor maps for one population buffer and its reference field: main-column boxes of
-// a single row and of TY rows.
+// Tensor maps for one population buffer and its reference field: boxes of 32 columns and 1,
+// 8 or 16 rows.
 struct TmaMaps {
-  CUtensorMap pop_main_row, pop_main_mid, pop_main_mid4;  // 32 columns, rows 1, 8, 4
-  CUtensorMap ref_main_row, ref_main_mid, ref_main_mid4;
-  CUtensorMap pop_w_row, pop_w_mid4, ref_w_row, ref_w_mid4;  // 64 columns, rows 1, 4 (nx % 64 == 0)
-  CUtensorMap pop_main_mid16, ref_main_mid16;                  // 32 columns, 16 rows (ny % 16 == 0)
-  bool mid16;                                                  // whether the last pair is encoded
+  CUtensorMap pop_main_row, pop_main_mid, pop_main_mid16;
+  CUtensorMap ref_main_row, ref_main_mid, ref_main_mid16;
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
