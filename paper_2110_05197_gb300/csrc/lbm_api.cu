@@ -50,6 +50,18 @@ bool is_device_ptr(const void* ptr) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// a pointer that kernels on the current device may write FP64 values through
+bool is_local_ptr(const void* ptr) {
+  if (!ptr || reinterpret_cast<uintptr_t>(ptr) % sizeof(double) != 0) return false;
+  cudaPointerAttributes a;
+  int dev = 0;
+  if (cudaPointerGetAttributes(&a, ptr) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
 lbm_status fail(lbm_ctx* c, cudaError_t e) {
   if (e == cudaSuccess) return LBM_OK;
   if (c->sticky == LBM_OK) c->sticky = LBM_ECUDA;
@@ -83,7 +95,7 @@ size_t workspace_layout(const lbm_params& p, lbm_ctx* c) {
   const long long N = (long long)p.nx * p.ny * p.nz;
   const size_t elt = p.precision == LBM_FP64 ? 8 : (p.precision == LBM_FP32 ? 4 : 2);
   const size_t relt = p.precision == LBM_FP64 ? 8 : 4;
-  const int nblk = (int)std::min<long long>((N + kDiagThreads - 1) / kDiagThreads, 1184);
+  const int nblk = (int)std::min<long long>((N + 63) / 64, 1184);
   size_t off = 0;
   auto take = [&](size_t b) {
     size_t o = off;
@@ -357,7 +369,7 @@ static lbm_status step_common(lbm_ctx* c, int32_t nsteps, bool cg) {
     c->cur ^= 1;
     c->steps += 1;
     if (c->p.diag_every > 0 && c->steps % c->p.diag_every == 0) {
-      e = lbm::launch_diagnostics(c, nullptr, false);
+      e = lbm::launch_diagnostics(c, nullptr, nullptr, nullptr, false);
       if (e != cudaSuccess) return fail(c, e);
     }
   }
@@ -376,12 +388,26 @@ lbm_status lbm_moments(lbm_ctx* c, double* rho_r, double* rho_b, double* u, doub
   cudaError_t e = cudaSuccess;
   const bool need_diag = rho_r || rho_b || u || totals;
   if (need_diag) {
-    double* u_dev = (u && is_device_ptr(u)) ? u : nullptr;
-    e = lbm::launch_diagnostics(c, u_dev, u != nullptr);
+    // results go straight to the caller's device buffers, or by way of the staging area; a
+    // device buffer of another GPU, or two that overlap, are filled by copies
+    const double* given[3] = {rho_r, rho_b, u};
+    const long long len[3] = {N, N, 3 * N};
+    bool direct[3], apart = true;
+    for (int i = 0; i < 3; i++) {
+      direct[i] = is_local_ptr(given[i]);
+      for (int k = 0; k < i; k++)
+        if (given[i] && given[k])
+          apart &= (uintptr_t)(given[i] + len[i]) <= (uintptr_t)given[k] || (uintptr_t)(given[k] + len[k]) <= (uintptr_t)given[i];
+    }
+    double* to[3] = {c->stage, c->stage + N, c->stage + 2 * N};
+    if (direct[0] && apart) to[0] = rho_r;
+    if (direct[1] && apart) to[1] = rho_b;
+    if (u && is_device_ptr(u)) to[2] = u;
+    e = lbm::launch_diagnostics(c, to[0], rho_b || c->K == 2 ? to[1] : nullptr, u ? to[2] : nullptr, totals != nullptr);
     if (e != cudaSuccess) return fail(c, e);
-    if (rho_r) e = copy_out(c, rho_r, c->stage, N * sizeof(double), &host);
-    if (e == cudaSuccess && rho_b) e = copy_out(c, rho_b, c->stage + N, N * sizeof(double), &host);
-    if (e == cudaSuccess && u && !u_dev) e = copy_out(c, u, c->stage + 2 * N, 3 * N * sizeof(double), &host);
+    if (rho_r && to[0] != rho_r) e = copy_out(c, rho_r, to[0], N * sizeof(double), &host);
+    if (e == cudaSuccess && rho_b && to[1] != rho_b) e = copy_out(c, rho_b, to[1], N * sizeof(double), &host);
+    if (e == cudaSuccess && u && to[2] != u) e = copy_out(c, u, to[2], 3 * N * sizeof(double), &host);
     if (e != cudaSuccess) return fail(c, e);
   }
   if (pops) {

@@ -46,8 +46,9 @@ struct AuxParams {
   int model, enhanced, K;
   double phi[2][3];      // rest-state weights per component and group
   double nu_r, nu_b;
-  double G, rho0;        // SC two-component: G = G_eff
+  double G, rho0, irho0; // SC two-component: G = G_eff; irho0 = 1 / rho0
   double body[3];
+  int forced;            // body is not 0
   double umax, neg_tol;
   double Ga[2], Gr[2];   // multirange SC self-couplings
   int px;                // row pitch and size of the stored arrays
@@ -77,7 +78,9 @@ AuxParams aux_params(const lbm_ctx* c) {
     a.Gr[k] = q.Gr[k];
   }
   a.rho0 = q.rho0_psi;
+  a.irho0 = 1.0 / q.rho0_psi;
   for (int d = 0; d < 3; d++) a.body[d] = q.body_force[d];
+  a.forced = a.body[0] != 0 || a.body[1] != 0 || a.body[2] != 0;
   a.umax = q.umax_unstable > 0 ? q.umax_unstable : 0.5;
   double scale = 1.0;
   if (q.model == LBM_MODEL_CG) scale = fmax(scale, fmax(q.rho_r0, q.rho_b0));
@@ -94,29 +97,75 @@ __device__ __forceinline__ int state_index(const lbm_diag* d, int cur) { return 
 template <class S>
 using step_t = typename std::conditional<std::is_same<S, double>::value, double, float>::type;
 
-// Sum of values of the compute type C whose FP64 result is as accurate as FP64 summation.
-// For C = float the sum is carried as an unevaluated pair s + c and the rounding error of
-// every addition is kept exactly (TwoSum), at FP32 cost: GB300's FP64 rate is a small
-// fraction of its FP32 rate, and the reductions here would otherwise be FP64 bound.
+// a value of the compute type in FP64, in integer arithmetic: GB300 runs conversions to FP64
+// at its low FP64 rate.  The exponent moves by 1023 - 127 (Inf and NaN: by 2047 - 255); a
+// subnormal is scaled to a normal number first.
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v) {
+  const bool sub = (__float_as_uint(v) & 0x7f800000u) == 0;
+  const unsigned b = __float_as_uint(sub ? v * 0x1p64f : v), m = b & 0x7fffffffu;
+  const unsigned up = sub ? 0x34000000u : m >= 0x7f800000u ? 0x70000000u : 0x38000000u;
+  return __hiloint2double(int((b & 0x80000000u) | (m == 0 ? 0 : (m >> 3) + up)), int(b << 29));
+}
+
+// The nodes a thread of densities_kernel handles at a time: two in FP32, whose packed
+// instructions work on both (lbm_vec.cuh), one in FP64.
 template <class C>
+struct Lanes;
+template <>
+struct Lanes<float> {
+  using V = F2;
+  static constexpr int W = 2;
+};
+template <>
+struct Lanes<double> {
+  using V = double;
+  static constexpr int W = 1;
+};
+__device__ __forceinline__ double lane(double v, int) { return v; }
+__device__ __forceinline__ float lane(const F2& v, int j) { return v[j]; }
+__device__ __forceinline__ void set_lane(double& v, int, double x) { v = x; }
+__device__ __forceinline__ void set_lane(F2& v, int j, float x) { v.set(j, x); }
+
+// Sum of values of the compute type whose FP64 result is as accurate as FP64 summation.  In
+// FP32 the sum is carried as an unevaluated pair s + c and the rounding error of every
+// addition is kept exactly (TwoSum), at FP32 cost: GB300's FP64 rate is a small fraction of
+// its FP32 rate, and the reductions here would otherwise be FP64 bound.
+template <class V>
 struct ExactSum;
 template <>
 struct ExactSum<double> {
-  double s = 0.0;
-  __device__ explicit ExactSum(double v = 0.0) : s(v) {}
-  __device__ void add(double v) { s += v; }
-  __device__ double value() const { return s; }
+  double s;
+  __device__ __forceinline__ explicit ExactSum(double v = 0.0) : s(v) {}
+  __device__ __forceinline__ void add(double v) { s += v; }
+  __device__ __forceinline__ void sub(double v) { s -= v; }
+  __device__ __forceinline__ void add(const ExactSum& o) { s += o.s; }
+  __device__ __forceinline__ void sub(const ExactSum& o) { s -= o.s; }
+  __device__ __forceinline__ double value(int) const { return s; }
 };
 template <>
-struct ExactSum<float> {
-  float s = 0.f, c = 0.f;
-  __device__ explicit ExactSum(float v = 0.f) : s(v) {}
-  __device__ void add(float v) {
-    float e;
-    s = two_sum(s, v, e);
-    c += e;
+struct ExactSum<F2> {
+  F2 s, c;
+  __device__ __forceinline__ explicit ExactSum(F2 v = F2(0.f)) : s(v), c(0.f) {}
+  __device__ __forceinline__ void add(F2 v) {
+    F2 e;
+    s = two_sum2(s, v, e);
+    c = c + e;
   }
-  __device__ double value() const { return double(s) + double(c); }
+  __device__ __forceinline__ void sub(F2 v) {  // TwoSum of s and -v
+    const F2 t = s - v, bb = t - s;
+    c = c + ((s - (t - bb)) - (v + bb));
+    s = t;
+  }
+  __device__ __forceinline__ void add(const ExactSum& o) {
+    add(o.s);
+    c = c + o.c;
+  }
+  __device__ __forceinline__ void sub(const ExactSum& o) {
+    sub(o.s);
+    c = c - o.c;
+  }
+  __device__ __forceinline__ double value(int j) const { return widen(s[j]) + widen(c[j]); }
 };
 
 // x, y, z of node n
@@ -281,285 +330,477 @@ __global__ void aa_gather_kernel(const S* __restrict__ f, S* __restrict__ out, c
 }
 
 
-// One pass over the populations: the component densities rr, rb (FP64, as exact as FP64
-// summation), psi of Eq. pseudopotential (SC multiphase, FP64), the momentum
-// j = sum_k sum_i c_i f^k_i into jm [3][N] (FP64), and for the multirange model the
-// pseudopotentials Psi_s of both species in the step's compute type into mrpsi [2][N]
-// (read 92 times per node by the diagnostics' belt sums).
-template <class L, class S, class RT, class I>
-__global__ void densities_kernel(const S* __restrict__ f0, const S* __restrict__ f1, const RT* __restrict__ r0,
-                                 const RT* __restrict__ r1, const lbm_diag* __restrict__ d, int cur,
-                                 double* __restrict__ rr, double* __restrict__ rb, double* __restrict__ psi,
-                                 double* __restrict__ jm, step_t<S>* __restrict__ mrpsi, AuxParams a) {
-  using C = step_t<S>;
-  const int b = state_index(d, cur);
-  const S* f = b ? f1 : f0;
-  const RT* r = b ? r1 : r0;
-  const bool odd = a.aa && (b & 1);
-  const I N = I(a.n), NS = I(a.ns);
-  for (I m = blockIdx.x * I(blockDim.x) + threadIdx.x; m < N; m += I(gridDim.x) * blockDim.x) {
-    // momentum summed exactly (ExactSum): the colours' momenta nearly cancel at
-    // interfaces, so rounding in the sum would show up in the reported u; the shift
-    // phi_i r is symmetric in c_i and carries no momentum: opposite pairs of the stored
-    // deviations
-    ExactSum<C> jx, jy, jz;
-    const I st = stored_index(m, a.nx, a.px);
-    auto at = [&](int k, int i) -> I {
-      return odd ? aa_index_nt<L, I>(k, i, m, a.nx, a.ny, a.nz, N, odd) : I(k * L::Q + i) * NS + st;
-    };
-    for (int k = 0; k < 2; k++) {
-      double s = 0.0;
-      if (k < a.K) {
-        ExactSum<C> acc{static_cast<C>(r[I(k) * NS + st])};  // sum_i phi_i = 1
-#pragma unroll
-        for (int i = 0; i < L::Q; i++)
-          acc.add(ld_s<S, C>(f[at(k, i)]));
-        s = acc.value();
-#pragma unroll
-        for (int q = 0; q < L::NP; q++) {
-          const C vp = ld_s<S, C>(f[at(k, 2 * q + 1)]);
-          const C vm = ld_s<S, C>(f[at(k, 2 * q + 2)]);
-          if (L::pcx(q)) { jx.add(L::pcx(q) > 0 ? vp : -vp); jx.add(L::pcx(q) > 0 ? -vm : vm); }
-          if (L::pcy(q)) { jy.add(L::pcy(q) > 0 ? vp : -vp); jy.add(L::pcy(q) > 0 ? -vm : vm); }
-          if (L::pcz(q)) { jz.add(L::pcz(q) > 0 ? vp : -vp); jz.add(L::pcz(q) > 0 ? -vm : vm); }
-        }
-      }
-      (k == 0 ? rr : rb)[m] = s;
-      // Eq. pseudopotential, once per node (the force stencil reads it 18 times)
-      if (k == 0 && a.model == LBM_MODEL_SC_MP) psi[m] = a.rho0 * (1.0 - exp(-s / a.rho0));
-      if (mrpsi) {  // Psi_s = rho_0 (1 - exp(-rho_s / rho_0)) in the compute type
-        const C c0 = C(a.rho0), ic0 = C(1.0 / a.rho0);
-        mrpsi[I(k) * N + m] = c0 * (C(1) - exp(-C(s) * ic0));
-      }
-    }
-    jm[m] = jx.value();
-    jm[N + m] = jy.value();
-    jm[2 * N + m] = jz.value();
-  }
-}
-
 // x is finite: its exponent field is not all ones (integer test of the high word; GB300
 // runs FP64 compares at its low FP64 rate).
 __device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 
 // ---- fixed-order block reductions ----
+// Ordered 64-bit keys of FP64 values: signed integer comparison orders them (GB300 runs FP64
+// compares at its low FP64 rate).
+__device__ __forceinline__ long long key_of(double v) {
+  const long long b = __double_as_longlong(v);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+__device__ __forceinline__ double of_key(long long k) {
+  return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffLL));
+}
+constexpr long long kInfKey = 0x7ff0000000000000LL;
+
+// A thread's share of the totals.  SUMS false: only what the blow-up check looks at, for
+// callers that do not ask for the totals.
 struct Acc {
-  double v[LBM_NTOTALS];
+  double sum[6];             // mass_r, mass_b, momentum, kinetic energy
+  long long uu, minr, minb;  // keys of max |u|^2 and of the smallest densities
+  int bad;                   // nodes with a value that is not finite
 };
-// slots: 0 mass_r 1 mass_b 2-4 mom 5 ekin 6 max|u| 7 nonfinite 8 min rr 9 min rb
 __device__ __forceinline__ void acc_init(Acc& a) {
-  for (int s = 0; s < LBM_NTOTALS; s++) a.v[s] = 0.0;
-  a.v[8] = INFINITY;
-  a.v[9] = INFINITY;
+  for (int s = 0; s < 6; s++) a.sum[s] = 0.0;
+  a.uu = 0;
+  a.minr = a.minb = kInfKey;
+  a.bad = 0;
 }
+template <bool SUMS>
 __device__ __forceinline__ void acc_merge(Acc& a, const Acc& b) {
-  for (int s = 0; s < 6; s++) a.v[s] += b.v[s];
-  a.v[6] = fmax(a.v[6], b.v[6]);
-  a.v[7] += b.v[7];
-  a.v[8] = fmin(a.v[8], b.v[8]);
-  a.v[9] = fmin(a.v[9], b.v[9]);
+  if constexpr (SUMS)
+    for (int s = 0; s < 6; s++) a.sum[s] += b.sum[s];
+  a.uu = max(a.uu, b.uu);
+  a.minr = min(a.minr, b.minr);
+  a.minb = min(a.minb, b.minb);
+  a.bad += b.bad;
 }
+template <bool SUMS>
 __device__ void block_reduce(Acc& a) {
-  __shared__ double sh[kDiagThreads / 32][LBM_NTOTALS];
+  __shared__ Acc sh[kDiagThreads / 32];
   for (int off = 16; off > 0; off >>= 1) {
     Acc o;
-    for (int s = 0; s < LBM_NTOTALS; s++) o.v[s] = __shfl_xor_sync(0xffffffffu, a.v[s], off);
-    acc_merge(a, o);
+    if constexpr (SUMS)
+      for (int s = 0; s < 6; s++) o.sum[s] = __shfl_xor_sync(0xffffffffu, a.sum[s], off);
+    o.uu = __shfl_xor_sync(0xffffffffu, a.uu, off);
+    o.minr = __shfl_xor_sync(0xffffffffu, a.minr, off);
+    o.minb = __shfl_xor_sync(0xffffffffu, a.minb, off);
+    o.bad = __shfl_xor_sync(0xffffffffu, a.bad, off);
+    acc_merge<SUMS>(a, o);
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0)
-    for (int s = 0; s < LBM_NTOTALS; s++) sh[warp][s] = a.v[s];
+  if (lane == 0) sh[warp] = a;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); w++) {
-      Acc o;
-      for (int s = 0; s < LBM_NTOTALS; s++) o.v[s] = sh[w][s];
-      acc_merge(a, o);
-    }
-  }
+  if (threadIdx.x == 0)
+    for (int w = 1; w < (int)(blockDim.x >> 5); w++) acc_merge<SUMS>(a, sh[w]);
 }
 
 // Fixed-order reduction of the nblk block partials into the totals and the blow-up status
 // (all threads of one block take part).
+template <bool SUMS>
 __device__ void reduce_partials(const double* partials, int nblk, lbm_diag* d, int cur, const AuxParams& a) {
   Acc acc;
   acc_init(acc);
   for (int b = threadIdx.x; b < nblk; b += blockDim.x) {
+    const double* p = partials + b * LBM_NTOTALS;
     Acc o;
-    for (int s = 0; s < LBM_NTOTALS; s++) o.v[s] = __ldcg(&partials[b * LBM_NTOTALS + s]);
-    acc_merge(acc, o);
+    if constexpr (SUMS)
+      for (int s = 0; s < 6; s++) o.sum[s] = __ldcg(&p[s]);
+    o.uu = key_of(__ldcg(&p[6]));
+    o.bad = (int)__ldcg(&p[7]);
+    o.minr = key_of(__ldcg(&p[8]));
+    o.minb = key_of(__ldcg(&p[9]));
+    acc_merge<SUMS>(acc, o);
   }
-  block_reduce(acc);
+  __syncthreads();  // the block's own reduction is done with the shared array
+  block_reduce<SUMS>(acc);
   if (threadIdx.x == 0) {
-    acc.v[6] = sqrt(acc.v[6]);  // max |u| from max |u|^2 (sqrt is monotonic and correctly rounded)
+    // max |u| from max |u|^2 (sqrt is monotonic and correctly rounded)
+    const double um = sqrt(of_key(acc.uu)), minr = of_key(acc.minr), minb = of_key(acc.minb);
     int st = 0;
-    if (acc.v[7] > 0 || !isfinite(acc.v[0]) || !isfinite(acc.v[1])) st |= 1;
-    if (acc.v[8] < -a.neg_tol || acc.v[9] < -a.neg_tol) st |= 2;
-    if (!(acc.v[6] <= a.umax)) st |= 4;
-    for (int s = 0; s < LBM_NTOTALS; s++) d->totals[s] = acc.v[s];
+    if (acc.bad > 0) st |= 1;
+    if constexpr (SUMS)
+      if (!isfinite(acc.sum[0]) || !isfinite(acc.sum[1])) st |= 1;
+    if (minr < -a.neg_tol || minb < -a.neg_tol) st |= 2;
+    if (!(um <= a.umax)) st |= 4;
+    if constexpr (SUMS)
+      for (int s = 0; s < 6; s++) d->totals[s] = acc.sum[s];
+    d->totals[6] = um;
+    d->totals[7] = acc.bad;
+    d->totals[8] = minr;
+    d->totals[9] = minb;
     if (d->status == 0 && st != 0) d->trip_buf = cur;
     d->status |= st;
   }
 }
 
-// Per-node velocity and the block partials of the totals, from the staged densities and
-// momentum (densities_kernel): no population is read again.  u (force-shifted, Eq.
-// guoforce) may be written over jm (uo == jm): each node reads its own momentum first.
-// Slot 6 of the partials holds max |u|^2 (its square root is taken in the final pass).
-template <class L, class S, class RT>
-__global__ void __launch_bounds__(kDiagThreads) diag_kernel(const double* __restrict__ rr,
-                                                            const double* __restrict__ rb,
-                                                            const double* __restrict__ psi,
-                                                            const double* jm,
-                                                            const step_t<S>* __restrict__ mrpsi,
-                                                            const uint8_t* __restrict__ solid, double* uo,
-                                                            double* __restrict__ partials, AuxParams a,
-                                                            const step_t<S>* __restrict__ colour,
-                                                            const step_t<S>* __restrict__ normals, RepParams rp,
-                                                            lbm_diag* __restrict__ d, int cur) {
-  using C = step_t<S>;  // per-node arithmetic of the multirange belts; the sums below are FP64
-  Acc acc;
-  acc_init(acc);
-  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < a.n; n += (long long)gridDim.x * blockDim.x) {
-    const bool wall = solid && solid[n];
-    const double j[3] = {jm[n], jm[a.n + n], jm[2 * a.n + n]};
-    const double r = rr[n], b = rb[n], rho = r + b;
-    const int bad = !(finite_bits(r) && finite_bits(b) && finite_bits(j[0]) && finite_bits(j[1]) && finite_bits(j[2]));
-    double F[3] = {a.body[0], a.body[1], a.body[2]};
-    if (!wall && a.model == LBM_MODEL_CG && normals) {
-      int x, y, z;
-      node_xyz(n, a, x, y, z);
-      C Fr[3];
-      rep_force<L, C>(normals, colour, solid, x, y, z, rp, Fr);  // the step's own precision
-      for (int dd = 0; dd < 3; dd++) F[dd] += double(Fr[dd]);
-    }
-    if (!wall && a.model != LBM_MODEL_CG) {
-      int x, y, z;
-      node_xyz(n, a, x, y, z);
-      // sum_i w_i phi(x + c_i) c_i as opposite-pair differences in FP64 (the force is a
-      // small difference of O(1) values); neighbour indices in 32-bit arithmetic when the
-      // node count allows it
-      double s1[3] = {0.0, 0.0, 0.0}, s2[3] = {0.0, 0.0, 0.0};
-      const double psic = a.model == LBM_MODEL_SC_MP ? psi[n] : 0.0;
-      const bool small = a.n < (1LL << 31);
-      const int xm = x == 0 ? a.nx - 1 : x - 1, xp = x + 1 == a.nx ? 0 : x + 1;
-      const int ym = y == 0 ? a.ny - 1 : y - 1, yp = y + 1 == a.ny ? 0 : y + 1;
-      const int zm = z == 0 ? a.nz - 1 : z - 1, zp = z + 1 == a.nz ? 0 : z + 1;
-      auto nbi = [&](int dx, int dy, int dz) -> long long {
-        const int X = dx == 0 ? x : (dx > 0 ? xp : xm);
-        const int Y = dy == 0 ? y : (dy > 0 ? yp : ym);
-        const int Z = dz == 0 ? z : (dz > 0 ? zp : zm);
-        return small ? (long long)(unsigned)(X + a.nx * (Y + a.ny * Z))
-                     : X + (long long)a.nx * (Y + (long long)a.ny * Z);
-      };
-#pragma unroll
-      for (int q = 0; q < L::NP; q++) {
-        const int i = 2 * q + 1;
-        const long long mp = nbi(cx<L>(i), cy<L>(i), cz<L>(i));
-        const long long mm = nbi(-cx<L>(i), -cy<L>(i), -cz<L>(i));
-        const bool swp = solid && solid[mp], swm = solid && solid[mm];
-        const double w = L::w(L::pgrp(q));
-        double d1, d2 = 0.0;
-        if (a.model == LBM_MODEL_SC_MP) {
-          d1 = w * ((swp ? psic : psi[mp]) - (swm ? psic : psi[mm]));
-        } else {
-          d1 = w * ((swp ? b : rb[mp]) - (swm ? b : rb[mm]));
-          d2 = w * ((swp ? r : rr[mp]) - (swm ? r : rr[mm]));
-        }
-        if (L::pcx(q)) { s1[0] += L::pcx(q) * d1; s2[0] += L::pcx(q) * d2; }
-        if (L::pcy(q)) { s1[1] += L::pcy(q) * d1; s2[1] += L::pcy(q) * d2; }
-        if (L::pcz(q)) { s1[2] += L::pcz(q) * d1; s2[2] += L::pcz(q) * d2; }
-      }
-      for (int dd = 0; dd < 3; dd++) {
-        if (a.model == LBM_MODEL_SC_MP)
-          F[dd] = -a.G * psic * s1[dd] + a.body[dd];
-        else
-          F[dd] = -a.G * r * s1[dd] - a.G * b * s2[dd] + a.body[dd];
-      }
-      if (a.model == LBM_MODEL_SC_MR) {
-        // self forces of Eqs. doublebeltattractiveforce / doublebeltrepulsionforce with
-        // the staged Psi_s, summed in the step's compute type C as the step kernel sums
-        // them (FP64 only for FP64 storage); a wall neighbour takes the centre value
-        const bool small = a.n < (1LL << 31);
-        for (int sp = 0; sp < 2; sp++) {
-          const C* ps = mrpsi + (long long)sp * a.n;
-          const C pc = ps[n];
-          auto psi_at = [&](int dx, int dy, int dz) -> C {
-            int X = x + dx, Y = y + dy, Z = z + dz;
-            X = X < 0 ? X + a.nx : (X >= a.nx ? X - a.nx : X);
-            Y = Y < 0 ? Y + a.ny : (Y >= a.ny ? Y - a.ny : Y);
-            Z = Z < 0 ? Z + a.nz : (Z >= a.nz ? Z - a.nz : Z);
-            const long long m = small ? (long long)(unsigned)(X + a.nx * (Y + a.ny * Z))
-                                      : X + (long long)a.nx * (Y + (long long)a.ny * Z);
-            return (solid && solid[m]) ? pc : ps[m];
-          };
-          C att[3] = {C(0), C(0), C(0)}, rep[3] = {C(0), C(0), C(0)};
-#pragma unroll
-          for (int q = 0; q < L::NP; q++) {
-            const C d = C(L::w(L::pgrp(q))) * (psi_at(L::pcx(q), L::pcy(q), L::pcz(q)) -
-                                               psi_at(-L::pcx(q), -L::pcy(q), -L::pcz(q)));
-            if (L::pcx(q)) att[0] += L::pcx(q) * d;
-            if (L::pcy(q)) att[1] += L::pcy(q) * d;
-            if (L::pcz(q)) att[2] += L::pcz(q) * d;
-          }
-#pragma unroll
-          for (int dz = 0; dz <= 2; dz++)
-#pragma unroll
-            for (int dy = -2; dy <= 2; dy++)
-#pragma unroll
-              for (int dx = -2; dx <= 2; dx++) {
-                const int r2 = dx * dx + dy * dy + dz * dz;
-                if (r2 == 0 || r2 > 8 || mr_weight(r2) == 0.0 || !(dz > 0 || dy > 0 || (dy == 0 && dx > 0))) continue;
-                const C d = C(mr_weight(r2)) * (psi_at(dx, dy, dz) - psi_at(-dx, -dy, -dz));
-                if (dx) rep[0] += C(dx) * d;
-                if (dy) rep[1] += C(dy) * d;
-                if (dz) rep[2] += C(dz) * d;
-              }
-          for (int dd = 0; dd < 3; dd++)
-            F[dd] += -a.Ga[sp] * double(pc) * double(att[dd]) - a.Gr[sp] * double(pc) * double(rep[dd]);
-        }
-      }
-    }
-    double u[3] = {0.0, 0.0, 0.0};
-    if (!wall) {
-      const double inv = 1.0 / rho;
-      for (int dd = 0; dd < 3; dd++) u[dd] = (j[dd] + 0.5 * F[dd]) * inv;
-    }
-    if (uo) {
-      uo[n] = u[0];
-      uo[a.n + n] = u[1];
-      uo[2 * a.n + n] = u[2];
-    }
-    if (wall) continue;
-    const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    acc.v[0] += r;
-    acc.v[1] += b;
-    acc.v[2] += j[0];
-    acc.v[3] += j[1];
-    acc.v[4] += j[2];
-    acc.v[5] += 0.5 * rho * uu;
-    acc.v[6] = fmax(acc.v[6], uu);
-    acc.v[7] += bad;
-    acc.v[8] = fmin(acc.v[8], r);
-    acc.v[9] = fmin(acc.v[9], b);
+// Velocity of one node (force-shifted, Eq. guoforce; 0 on walls) and its share of the totals.
+template <bool SUMS, bool FORCED = true>
+__device__ __forceinline__ void diag_node(bool wall, double r, double b, const double (&j)[3], const double (&F)[3],
+                                          double (&u)[3], Acc& acc) {
+  u[0] = u[1] = u[2] = 0.0;
+  if (wall) return;
+  const double rho = r + b;
+  const double inv = 1.0 / rho;
+  for (int t = 0; t < 3; t++) u[t] = (FORCED ? j[t] + 0.5 * F[t] : j[t]) * inv;
+  const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+  if constexpr (SUMS) {
+    acc.sum[0] += r;
+    acc.sum[1] += b;
+    acc.sum[2] += j[0];
+    acc.sum[3] += j[1];
+    acc.sum[4] += j[2];
+    acc.sum[5] += 0.5 * rho * uu;
   }
-  block_reduce(acc);
-  // The block that finishes last reduces every block's partial (in block order, whatever
-  // the finishing order): partial written, fence, count; the counter goes back to 0.
+  // fmax / fmin: a NaN does not count (its key is beyond the infinities')
+  const long long ku = key_of(uu), kr = key_of(r), kb = key_of(b);
+  if (ku <= kInfKey) acc.uu = max(acc.uu, ku);
+  if (kr >= ~kInfKey) acc.minr = min(acc.minr, kr);
+  if (kb >= ~kInfKey) acc.minb = min(acc.minb, kb);
+  acc.bad += !(finite_bits(r) && finite_bits(b) && finite_bits(j[0]) && finite_bits(j[1]) && finite_bits(j[2]));
+}
+
+// The block that finishes last reduces every block's partial (in block order, whatever the
+// finishing order): partial written, fence, count; the counter goes back to 0.  Slot 6 of
+// the partials holds max |u|^2 (its square root is taken in the final pass).
+template <bool SUMS>
+__device__ __forceinline__ void diag_finish(Acc& acc, double* __restrict__ partials, lbm_diag* __restrict__ d, int cur,
+                                            const AuxParams& a) {
+  block_reduce<SUMS>(acc);
   __shared__ bool last;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < LBM_NTOTALS; s++) partials[blockIdx.x * LBM_NTOTALS + s] = acc.v[s];
+    double* p = partials + blockIdx.x * LBM_NTOTALS;
+    if constexpr (SUMS)
+      for (int s = 0; s < 6; s++) p[s] = acc.sum[s];
+    p[6] = of_key(acc.uu);
+    p[7] = acc.bad;
+    p[8] = of_key(acc.minr);
+    p[9] = of_key(acc.minb);
     __threadfence();
     last = atomicAdd(&d->done, 1u) == gridDim.x - 1;
   }
   __syncthreads();
   if (last) {
     __threadfence();
-    reduce_partials(partials, gridDim.x, d, cur, a);
+    reduce_partials<SUMS>(partials, gridDim.x, d, cur, a);
     if (threadIdx.x == 0) d->done = 0;
   }
 }
 
+// One pass over the populations: the component densities rr, rb (FP64, as exact as FP64
+// summation), psi of Eq. pseudopotential (SC multiphase, FP64), the momentum
+// j = sum_k sum_i c_i f^k_i into jm [3][N] (FP64), and for the multirange model the
+// pseudopotentials Psi_s of both species in the step's compute type into mrpsi [2][N].
+// FUSED (no force that depends on other nodes): the velocity and the totals as well, so that
+// neither the densities nor the momentum are read again.
+// rb may be null with one component.  `pitch`/`rows`: stored rows of `row` nodes, `pitch`
+// apart (one row of N nodes where they are dense); vld: pairs of stored nodes are aligned;
+// vst: pairs of FP64 results are.
+// Bound by FP32 issue as scalar code: 128^3 CG FP32 107 us, with the reads of diag_kernel
+// 274; two nodes a thread and fused 115 us (403 MB: 59 us at the copy rate).
+template <class L, class S, class RT, int MODEL, bool FUSED, bool SUMS>
+__global__ void __launch_bounds__(kDiagThreads, 2) densities_kernel(
+    const S* __restrict__ f0, const S* __restrict__ f1, const RT* __restrict__ r0, const RT* __restrict__ r1,
+    lbm_diag* __restrict__ d, int cur, double* __restrict__ rr, double* __restrict__ rb, double* __restrict__ psi,
+    double* __restrict__ jm, step_t<S>* __restrict__ mrpsi, const uint8_t* __restrict__ solid,
+    double* __restrict__ partials, AuxParams a, unsigned row, unsigned pitch, unsigned rows, int vld, int vst) {
+  using C = step_t<S>;
+  using V = typename Lanes<C>::V;
+  constexpr int W = Lanes<C>::W, K = MODEL == LBM_MODEL_SC_MP ? 1 : 2;
+  const int b = state_index(d, cur);
+  const S* f = b ? f1 : f0;
+  const RT* r = b ? r1 : r0;
+  const bool odd = a.aa && (b & 1);
+  const unsigned per = (row + W - 1) / W, total = per * rows;
+  [[maybe_unused]] Acc acc;
+  if constexpr (FUSED) acc_init(acc);
+  for (unsigned p = blockIdx.x * blockDim.x + threadIdx.x; p < total; p += gridDim.x * blockDim.x) {
+    const unsigned y = rows == 1 ? 0 : p / per, x = (p - y * per) * W;
+    const unsigned n = y * row + x, st = y * pitch + x;
+    const bool two = W == 1 || x + 1 < row;  // else the second node is beyond the row's end
+    auto load = [&](auto* arr) -> V {  // of a stored array
+      using E = typename std::remove_const<typename std::remove_pointer<decltype(arr)>::type>::type;
+      V v;
+      if constexpr (W == 1) {
+        v = ld_s<E, C>(arr[st]);
+      } else {
+        E e[2];
+        if (vld) {
+          using U = typename std::conditional<sizeof(E) == 4, uint2, unsigned>::type;
+          *reinterpret_cast<U*>(e) = *reinterpret_cast<const U*>(arr + st);
+        } else {
+          e[0] = arr[st];
+          e[1] = two ? arr[st + 1] : e[0];
+        }
+        v.set(0, ld_s<E, C>(e[0]));
+        v.set(1, ld_s<E, C>(e[1]));
+      }
+      return v;
+    };
+    // the shift phi_i r is symmetric in c_i and carries no momentum: opposite pairs of the
+    // stored deviations.  The colours' momenta nearly cancel at interfaces, so rounding in
+    // the sum would show up in the reported u: exact sums
+    ExactSum<V> j[3], s[K];
+#pragma unroll
+    for (int k = 0; k < K; k++) {
+      V g[L::Q];
+      if (odd) {
+#pragma unroll
+        for (int i = 0; i < L::Q; i++)
+#pragma unroll
+          for (int l = 0; l < W; l++)
+            set_lane(g[i], l, ld_s<S, C>(f[aa_index_n<L>(k, i, l && two ? n + l : n, a.nx, a.ny, a.nz, a.n, true)]));
+      } else {
+#pragma unroll
+        for (int i = 0; i < L::Q; i++) g[i] = load(f + (k * L::Q + i) * a.ns);
+      }
+      s[k] = ExactSum<V>(load(r + k * a.ns));  // sum_i phi_i = 1
+#pragma unroll
+      for (int i = 0; i < L::Q; i++) s[k].add(g[i]);
+#pragma unroll
+      for (int q = 0; q < L::NP; q++) {
+        ExactSum<V> dq(g[2 * q + 1]);
+        dq.sub(g[2 * q + 2]);
+        const int c[3] = {L::pcx(q), L::pcy(q), L::pcz(q)};
+#pragma unroll
+        for (int t = 0; t < 3; t++)
+          if (c[t] > 0) j[t].add(dq); else if (c[t] < 0) j[t].sub(dq);
+      }
+    }
+    double out[5][W];  // rr, rb, j or u
+#pragma unroll
+    for (int l = 0; l < W; l++) {
+      out[0][l] = s[0].value(l);
+      out[1][l] = K == 2 ? s[K - 1].value(l) : 0.0;
+      const double jj[3] = {j[0].value(l), j[1].value(l), j[2].value(l)};
+      for (int t = 0; t < 3; t++) out[2 + t][l] = jj[t];
+      if (l && !two) break;
+      if constexpr (FUSED) {
+        const double F[3] = {a.body[0], a.body[1], a.body[2]};
+        double u[3];
+        const bool wall = solid && solid[n + l];
+        if (a.forced)
+          diag_node<SUMS>(wall, out[0][l], out[1][l], jj, F, u, acc);
+        else
+          diag_node<SUMS, false>(wall, out[0][l], out[1][l], jj, F, u, acc);
+        for (int t = 0; t < 3; t++) out[2 + t][l] = u[t];
+      }
+      // Eq. pseudopotential, once per node (the force stencil reads it 18 times)
+      if constexpr (MODEL == LBM_MODEL_SC_MP) psi[n + l] = a.rho0 * (1.0 - exp(-out[0][l] * a.irho0));
+      if constexpr (MODEL == LBM_MODEL_SC_MR) {  // Psi_s = rho_0 (1 - exp(-rho_s / rho_0)) in the compute type
+        const C c0 = C(a.rho0), ic0 = C(a.irho0);
+        for (int k = 0; k < 2; k++) mrpsi[k * a.n + n + l] = c0 * (C(1) - exp(-C(out[k][l]) * ic0));
+      }
+    }
+    double* const dst[5] = {rr, rb, jm, jm + a.n, jm + 2 * a.n};
+#pragma unroll
+    for (int t = 0; t < 5; t++) {
+      if ((t == 1 && K == 1 && !rb) || (FUSED && t >= 2 && !jm)) continue;
+      if (W == 2 && vst && two) {
+        *reinterpret_cast<double2*>(dst[t] + n) = make_double2(out[t][0], out[t][W - 1]);
+      } else {
+        dst[t][n] = out[t][0];
+        if (W == 2 && two) dst[t][n + 1] = out[t][W - 1];
+      }
+    }
+  }
+  if constexpr (FUSED) diag_finish<SUMS>(acc, partials, d, cur, a);
+}
+
+// Index of the neighbour of (x, y, z), all steps at most 2 with one periodic wrap.  32-bit: no
+// device holds the workspace of 2^32 nodes.
+__device__ __forceinline__ unsigned wrapped(int x, int y, int z, const AuxParams& a) {
+  x = x < 0 ? x + a.nx : (x >= a.nx ? x - a.nx : x);
+  y = y < 0 ? y + a.ny : (y >= a.ny ? y - a.ny : y);
+  z = z < 0 ? z + a.nz : (z >= a.nz ? z - a.nz : z);
+  return unsigned(x) + unsigned(a.nx) * (unsigned(y) + unsigned(a.ny) * unsigned(z));
+}
+
+// sum_i w_i phi(x + c_i) c_i of one field as opposite-pair differences in FP64 (the force is
+// a small difference of O(1) values), in units of the diagonal weight: the axis differences
+// weigh w_axis / w_diagonal times as much, so that a component takes one product.
+template <class L>
+struct Gradient {
+  double s[3] = {0.0, 0.0, 0.0};
+  double ax[3] = {0.0, 0.0, 0.0};
+  __device__ __forceinline__ void add(int q, double dq) {
+    const int c[3] = {L::pcx(q), L::pcy(q), L::pcz(q)};
+#pragma unroll
+    for (int t = 0; t < 3; t++) {
+      if (c[t] == 0) continue;
+      if (L::pgrp(q) == 1) ax[t] = dq;
+      else if (c[t] > 0) s[t] += dq;
+      else s[t] -= dq;
+    }
+  }
+  __device__ __forceinline__ double at(int t) const {
+    constexpr double ratio = L::D == 3 ? 2.0 : 4.0;  // w(1) / w(2), exact
+    return ratio * ax[t] + s[t];
+  }
+};
+
+// F = body - G (r grad b + b grad r) or body - G psi grad psi, of one node
+template <class L, int MODEL, bool WALLS>
+__device__ __forceinline__ void sc_force(const double* __restrict__ rr, const double* __restrict__ rb,
+                                         const double* __restrict__ psi, const uint8_t* __restrict__ solid, double r,
+                                         double b, unsigned n, int x, int y, int z, const AuxParams& a, double (&F)[3]) {
+  Gradient<L> g1, g2;
+  const double pc = MODEL == LBM_MODEL_SC_MP ? psi[n] : 0.0;
+#pragma unroll
+  for (int q = 0; q < L::NP; q++) {
+    const unsigned mp = wrapped(x + L::pcx(q), y + L::pcy(q), z + L::pcz(q), a);
+    const unsigned mm = wrapped(x - L::pcx(q), y - L::pcy(q), z - L::pcz(q), a);
+    const bool wp = WALLS && solid[mp], wm = WALLS && solid[mm];
+    if constexpr (MODEL == LBM_MODEL_SC_MP) {
+      g1.add(q, (wp ? pc : psi[mp]) - (wm ? pc : psi[mm]));
+    } else {
+      g1.add(q, (wp ? b : rb[mp]) - (wm ? b : rb[mm]));
+      g2.add(q, (wp ? r : rr[mp]) - (wm ? r : rr[mm]));
+    }
+  }
+  const double gw = -a.G * L::w(2);
+  if constexpr (MODEL == LBM_MODEL_SC_MP) {
+    const double gp = gw * pc;
+    for (int t = 0; t < 3; t++) F[t] = gp * g1.at(t) + a.body[t];
+  } else {
+    const double gr = gw * r, gb = gw * b;
+    for (int t = 0; t < 3; t++) F[t] = gr * g1.at(t) + (gb * g2.at(t) + a.body[t]);
+  }
+}
+
+// Per-node velocity and the block partials of the totals, from the staged densities and
+// momentum (densities_kernel): no population is read again.  u (force-shifted, Eq.
+// guoforce) may be written over jm (uo == jm): each node reads its own momentum first.
+// FP64 issue bounds it (2 operations per clock and SM): every factor common to a stencil is
+// applied once to its sum.  128^3 SC multiphase 339 -> 183 us, two components 442 ->
+// 290 us.
+template <class L, class C, int MODEL, bool WALLS, bool SUMS>
+__global__ void __launch_bounds__(kDiagThreads) diag_kernel(const double* __restrict__ rr,
+                                                            const double* __restrict__ rb,
+                                                            const double* __restrict__ psi,
+                                                            const double* jm, const uint8_t* __restrict__ solid,
+                                                            double* uo, double* __restrict__ partials, AuxParams a,
+                                                            const C* __restrict__ colour,
+                                                            const C* __restrict__ normals, RepParams rp,
+                                                            lbm_diag* __restrict__ d, int cur) {
+  Acc acc;
+  acc_init(acc);
+  const unsigned N = (unsigned)a.n;
+  for (unsigned n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += gridDim.x * blockDim.x) {
+    const bool wall = WALLS && solid[n];
+    const double j[3] = {jm[n], jm[a.n + n], jm[2 * a.n + n]};
+    const double r = rr[n], b = MODEL == LBM_MODEL_SC_MP ? 0.0 : rb[n];
+    double F[3] = {a.body[0], a.body[1], a.body[2]};
+    if (!wall) {
+      int x, y, z;
+      node_xyz(n, a, x, y, z);
+      if constexpr (MODEL == LBM_MODEL_CG) {  // repulsion
+        C Fr[3];
+        rep_force<L, C>(normals, colour, WALLS ? solid : nullptr, x, y, z, rp, Fr);  // the step's own precision
+        for (int t = 0; t < 3; t++) F[t] += widen(Fr[t]);
+      } else {
+        sc_force<L, MODEL, WALLS>(rr, rb, psi, solid, r, b, n, x, y, z, a, F);
+      }
+    }
+    double u[3];
+    diag_node<SUMS>(wall, r, b, j, F, u, acc);
+    if (uo)
+      for (int t = 0; t < 3; t++) uo[t * a.n + n] = u[t];
+  }
+  diag_finish<SUMS>(acc, partials, d, cur, a);
+}
+
+// The same for the multirange model: self forces of Eqs. doublebeltattractiveforce /
+// doublebeltrepulsionforce with the staged Psi_s, summed in the step's compute type C as the
+// step kernel sums them; a wall neighbour takes the centre value.  Each node reads 92 values
+// of either species: a block marches along z over a tile of 32 x 8 nodes with the five
+// planes around it in shared memory (two halo nodes).  128x64x64: 674 us with the neighbours
+// gathered from global memory, 121 us from the planes (FP64 issue of the
+// cross force bounds it).
+constexpr int kMrTX = 32, kMrTY = kDiagThreads / kMrTX, kMrEX = kMrTX + 4, kMrEY = kMrTY + 4, kMrZ = 4;
+template <class C, bool WALLS, bool SUMS>
+__global__ void __launch_bounds__(kDiagThreads) diag_mr_kernel(const double* __restrict__ rr,
+                                                               const double* __restrict__ rb,
+                                                               const C* __restrict__ mrpsi, const double* jm,
+                                                               const uint8_t* __restrict__ solid, double* uo,
+                                                               double* __restrict__ partials, AuxParams a,
+                                                               lbm_diag* __restrict__ d, int cur) {
+  using L = D3Q19;
+  constexpr int NE = kMrEX * kMrEY;
+  __shared__ C ps[5][2][NE];
+  __shared__ uint8_t msk[5][WALLS ? NE : 1];
+  Acc acc;
+  acc_init(acc);
+  const int ncx = (a.nx + kMrTX - 1) / kMrTX, ncy = (a.ny + kMrTY - 1) / kMrTY, ncz = (a.nz + kMrZ - 1) / kMrZ;
+  const long long units = (long long)ncx * ncy * ncz;
+  const int tx = threadIdx.x % kMrTX, ty = threadIdx.x / kMrTX;
+  for (long long w = blockIdx.x; w < units; w += gridDim.x) {
+    const int bx = int(w % ncx) * kMrTX, by = int(w / ncx % ncy) * kMrTY, z0 = int(w / ncx / ncy) * kMrZ;
+    const int z1 = min(z0 + kMrZ, a.nz);
+    auto stage = [&](int z) {  // plane z into slot (z + 5) % 5; beyond the lattice, its periodic image
+      const int zw = ((z % a.nz) + a.nz) % a.nz, slot = (z + 5) % 5;
+      for (int e = threadIdx.x; e < NE; e += kDiagThreads) {
+        const int X = bx + e % kMrEX - 2, Y = by + e / kMrEX - 2;
+        const int Xw = (X + 2 * a.nx) % a.nx, Yw = (Y + 2 * a.ny) % a.ny;
+        const unsigned m = wrapped(Xw, Yw, zw, a);
+        ps[slot][0][e] = mrpsi[m];
+        ps[slot][1][e] = mrpsi[a.n + m];
+        if constexpr (WALLS) msk[slot][e] = solid[m];
+      }
+    };
+    __syncthreads();  // the last unit's reads are done
+    for (int z = z0 - 2; z < z0 + 2; z++) stage(z);
+    for (int z = z0; z < z1; z++) {
+      stage(z + 2);
+      __syncthreads();
+      const int x = bx + tx, y = by + ty;
+      if (x < a.nx && y < a.ny) {
+        const unsigned n = wrapped(x, y, z, a);
+        const bool wall = WALLS && solid[n];
+        const double j[3] = {jm[n], jm[a.n + n], jm[2 * a.n + n]};
+        const double r = rr[n], b = rb[n];
+        double F[3] = {a.body[0], a.body[1], a.body[2]};
+        if (!wall) {
+          sc_force<L, LBM_MODEL_SC_MR, WALLS>(rr, rb, nullptr, solid, r, b, n, x, y, z, a, F);
+          int slot[5];
+#pragma unroll
+          for (int t = 0; t < 5; t++) slot[t] = (z + t + 3) % 5;  // plane z + t - 2
+          const int e0 = (ty + 2) * kMrEX + tx + 2;
+#pragma unroll
+          for (int sp = 0; sp < 2; sp++) {
+            const C pc = ps[slot[2]][sp][e0];
+            auto psi_at = [&](int dx, int dy, int dz) -> C {
+              const int e = e0 + dy * kMrEX + dx, t = slot[dz + 2];
+              if (WALLS && msk[t][e]) return pc;
+              return ps[t][sp][e];
+            };
+            C att[3] = {C(0), C(0), C(0)}, rep[3] = {C(0), C(0), C(0)};
+#pragma unroll
+            for (int dz = 0; dz <= 2; dz++)
+#pragma unroll
+              for (int dy = -2; dy <= 2; dy++)
+#pragma unroll
+                for (int dx = -2; dx <= 2; dx++) {
+                  const int r2 = dx * dx + dy * dy + dz * dz;
+                  if (r2 == 0 || r2 > 8 || mr_weight(r2) == 0.0 || !(dz > 0 || dy > 0 || (dy == 0 && dx > 0))) continue;
+                  const C diff = psi_at(dx, dy, dz) - psi_at(-dx, -dy, -dz);
+                  const C dr = C(mr_weight(r2)) * diff;
+                  if (dx) rep[0] += C(dx) * dr;
+                  if (dy) rep[1] += C(dy) * dr;
+                  if (dz) rep[2] += C(dz) * dr;
+                  if (r2 > 2) continue;
+                  const C da = C(L::w(r2)) * diff;
+                  if (dx) att[0] += C(dx) * da;
+                  if (dy) att[1] += C(dy) * da;
+                  if (dz) att[2] += C(dz) * da;
+                }
+            const double ga = -a.Ga[sp] * widen(pc), gr = -a.Gr[sp] * widen(pc);
+            for (int t = 0; t < 3; t++) F[t] += ga * widen(att[t]) + gr * widen(rep[t]);
+          }
+        }
+        double u[3];
+        diag_node<SUMS>(wall, r, b, j, F, u, acc);
+        if (uo)
+          for (int t = 0; t < 3; t++) uo[t * a.n + n] = u[t];
+      }
+      __syncthreads();
+    }
+  }
+  diag_finish<SUMS>(acc, partials, d, cur, a);
+}
 
 // Which nodes are walls or have one beside them, and a list of the latter
 // (lbm_step_pair.cuh).
@@ -642,32 +883,72 @@ cudaError_t gather_t(lbm_ctx* c, void* out, int k, int i) {
   return cudaGetLastError();
 }
 
-template <class L, class S, class RT>
-cudaError_t diag_t(lbm_ctx* c, double* uo) {
+// Threads of a block of the moment kernels for `items` of work: fewer on small lattices, whose
+// FP64 work then spreads over all SMs (2D 128^2 CG FP64: 20.6 us with 256, 16.0 with this rule;
+// the same on lattices that fill the SMs either way).
+int diag_threads(const lbm_ctx* c, long long items) {
+  int t = kDiagThreads;
+  while (t > 64 && items < (long long)t * c->nsm) t /= 2;
+  return t;
+}
+
+template <class L, class S, class RT, int MODEL, bool FUSED, bool SUMS>
+cudaError_t densities_t(lbm_ctx* c, const AuxParams& a, double* rr, double* rb, double* psi, double* jm) {
+  using C = step_t<S>;
+  constexpr int W = Lanes<C>::W;
+  const bool dense = c->px == c->p.nx;
+  const long long row = dense ? c->N : c->p.nx, pitch = dense ? c->N : c->px, rows = c->N / row;
+  const long long total = (row + W - 1) / W * rows;
+  const int threads = diag_threads(c, total);
+  const int blocks = (int)std::min<long long>((total + threads - 1) / threads, FUSED ? 2 * c->nsm : c->nblk_diag);
+  // pairs are aligned where rows and whole arrays hold an even number of nodes
+  const int vld = pitch % 2 == 0 && c->NS % 2 == 0;
+  auto at16 = [](const double* p) { return !p || reinterpret_cast<uintptr_t>(p) % 16 == 0; };
+  const int vst = row % 2 == 0 && c->N % 2 == 0 && at16(rr) && at16(rb) && at16(jm);
+  C* mrpsi = MODEL == LBM_MODEL_SC_MR ? reinterpret_cast<C*>(psi) : nullptr;
+  const uint8_t* solid = c->has_walls ? c->solid : nullptr;
+  densities_kernel<L, S, RT, MODEL, FUSED, SUMS><<<blocks, threads, 0, c->stream>>>(
+      static_cast<const S*>(c->f[0]), static_cast<const S*>(c->f[1]), static_cast<const RT*>(c->r[0]),
+      static_cast<const RT*>(c->r[1]), c->diag, c->cur, rr, rb, psi, jm, mrpsi, solid, c->partials, a, (unsigned)row,
+      (unsigned)pitch, (unsigned)rows, vld, vst);
+  c->launches += 1;
+  return cudaGetLastError();
+}
+
+// rr, rb: where the densities go (rb null: a single component's, not asked for); uo: where
+// the velocity goes, null if it is not asked for.
+template <class L, class S, class RT, int MODEL, bool SUMS>
+cudaError_t diag_t(lbm_ctx* c, double* rr, double* rb, double* uo) {
+  using C = step_t<S>;
   const AuxParams a = aux_params(c);
-  const S* f0 = static_cast<const S*>(c->f[0]);
-  const S* f1 = static_cast<const S*>(c->f[1]);
-  const RT* r0 = static_cast<const RT*>(c->r[0]);
-  const RT* r1 = static_cast<const RT*>(c->r[1]);
-  double* rr = c->stage;
-  double* rb = c->stage + c->N;
   double* jm = c->stage + 2 * c->N;   // momentum, then (if requested here) the velocity
   double* psi = c->stage + 5 * c->N;  // SC multiphase psi (FP64), or the multirange Psi_s
-  step_t<S>* mrpsi = c->p.model == LBM_MODEL_SC_MR ? reinterpret_cast<step_t<S>*>(psi) : nullptr;
-  auto dens = (long long)c->K * c->Q * c->NS < (1LL << 31) ? densities_kernel<L, S, RT, int>
-                                                          : densities_kernel<L, S, RT, long long>;
-  dens<<<grid_for(c->N, 256, 8192), 256, 0, c->stream>>>(f0, f1, r0, r1, c->diag, c->cur, rr, rb, psi, jm, mrpsi, a);
-  cudaError_t e = cudaGetLastError();
+  const uint8_t* solid = c->has_walls ? c->solid : nullptr;
+  if constexpr (MODEL == LBM_MODEL_CG)
+    if (!c->rep) return densities_t<L, S, RT, MODEL, true, SUMS>(c, a, rr, rb, psi, uo);
+  cudaError_t e = densities_t<L, S, RT, MODEL, false, false>(c, a, rr, rb, psi, jm);
   if (e != cudaSuccess) return e;
-  if (c->rep) {
-    e = launch_rep_prepass_t<L, step_t<S>, S, RT>(c, c->cur);
-    if (e != cudaSuccess) return e;
+  if constexpr (MODEL == LBM_MODEL_SC_MR) {
+    auto kern = solid ? diag_mr_kernel<C, true, SUMS> : diag_mr_kernel<C, false, SUMS>;
+    const long long units = (long long)((c->p.nx + kMrTX - 1) / kMrTX) * ((c->p.ny + kMrTY - 1) / kMrTY) *
+                            ((c->p.nz + kMrZ - 1) / kMrZ);
+    kern<<<(int)std::min<long long>(units, c->nblk_diag), kDiagThreads, 0, c->stream>>>(
+        rr, rb, reinterpret_cast<const C*>(psi), jm, solid, uo, c->partials, a, c->diag, c->cur);
+  } else {
+    if (MODEL == LBM_MODEL_CG) {
+      e = launch_rep_prepass_t<L, C, S, RT>(c, c->cur);
+      if (e != cudaSuccess) return e;
+    }
+    // the SC forces do not depend on the compute type
+    using CK = typename std::conditional<MODEL == LBM_MODEL_CG, C, float>::type;
+    auto kern = solid ? diag_kernel<L, CK, MODEL, true, SUMS> : diag_kernel<L, CK, MODEL, false, SUMS>;
+    const int threads = diag_threads(c, c->N);
+    const int blocks = (int)std::min<long long>((c->N + threads - 1) / threads, c->nblk_diag);
+    kern<<<blocks, threads, 0, c->stream>>>(rr, rb, psi, jm, solid, uo, c->partials, a,
+                                                       static_cast<const CK*>(c->colour),
+                                                       static_cast<const CK*>(c->normals), rep_params(c), c->diag, c->cur);
   }
-  diag_kernel<L, S, RT><<<c->nblk_diag, kDiagThreads, 0, c->stream>>>(
-      rr, rb, psi, jm, mrpsi, c->has_walls ? c->solid : nullptr, uo, c->partials, a,
-      static_cast<const step_t<S>*>(c->colour), static_cast<const step_t<S>*>(c->normals), rep_params(c), c->diag,
-      c->cur);
-  c->launches += 2;
+  c->launches += 1;
   return cudaGetLastError();
 }
 
@@ -709,7 +990,25 @@ struct GatherOp {
 };
 template <class L, class S, class RT>
 struct DiagOp {
-  static cudaError_t run(lbm_ctx* c, double* uo) { return diag_t<L, S, RT>(c, uo); }
+  static cudaError_t run(lbm_ctx* c, double* rr, double* rb, double* uo, bool totals) {
+    // FP64 densities can overflow their sum, which the blow-up check looks at: always summed
+    if (totals || std::is_same<S, double>::value) return by_model<true>(c, rr, rb, uo);
+    return by_model<false>(c, rr, rb, uo);
+  }
+  template <bool SUMS>
+  static cudaError_t by_model(lbm_ctx* c, double* rr, double* rb, double* uo) {
+    switch (c->p.model) {
+      case LBM_MODEL_CG:
+        return diag_t<L, S, RT, LBM_MODEL_CG, SUMS>(c, rr, rb, uo);
+      case LBM_MODEL_SC_MP:
+        return diag_t<L, S, RT, LBM_MODEL_SC_MP, SUMS>(c, rr, rb, uo);
+      case LBM_MODEL_SC_2C:
+        return diag_t<L, S, RT, LBM_MODEL_SC_2C, SUMS>(c, rr, rb, uo);
+      default:
+        if constexpr (L::D == 3) return diag_t<L, S, RT, LBM_MODEL_SC_MR, SUMS>(c, rr, rb, uo);
+        return cudaErrorInvalidValue;
+    }
+  }
 };
 
 }  // namespace
@@ -753,9 +1052,10 @@ cudaError_t launch_aa_gather_plane(lbm_ctx* c, void* out, int k, int i) {
   return by_lattice_precision<GatherOp>(c, out, k, i);
 }
 
-cudaError_t launch_diagnostics(lbm_ctx* c, double* u_out, bool want_u) {
-  double* uo = u_out ? u_out : (want_u ? c->stage + 2 * c->N : nullptr);
-  return by_lattice_precision<DiagOp>(c, uo);
+cudaError_t launch_diagnostics(lbm_ctx* c, double* rho_r, double* rho_b, double* u_out, bool totals) {
+  if (!rho_r) rho_r = c->stage;
+  if (!rho_b && c->K == 2) rho_b = c->stage + c->N;
+  return by_lattice_precision<DiagOp>(c, rho_r, rho_b, u_out, totals);
 }
 
 }  // namespace lbm

@@ -112,9 +112,10 @@ cudaError_t launch_export_all(lbm_ctx* c, double* pops);
 // In-place streaming at odd parity: stored plane (k, i) of the even layout into out [N]
 // (storage type), i.e. slot opp(i) of node x - c_i for every x.
 cudaError_t launch_aa_gather_plane(lbm_ctx* c, void* out, int k, int i);
-// Densities into stage[0..2N), velocity into u_out (or stage[2N..5N) when null and
-// want_u), block partials, then the fixed-order final reduction into c->diag.
-cudaError_t launch_diagnostics(lbm_ctx* c, double* u_out, bool want_u);
+// Densities into rho_r, rho_b (null: the staging area; a single component's rho_b is then
+// left out), velocity into u_out unless that is null, the blow-up status and, if asked for,
+// the totals into the diagnostics record.
+cudaError_t launch_diagnostics(lbm_ctx* c, double* rho_r, double* rho_b, double* u_out, bool totals);
 // Repulsion pre-pass (colour and normal fields) of the current state, for the diagnostics.
 cudaError_t launch_rep_prepass(lbm_ctx* c);
 
