@@ -145,7 +145,7 @@ size_t workspace_layout(const lbm_params& p, lbm_ctx* c) {
     c->diag = reinterpret_cast<lbm_diag*>(c->ws + odia);
     c->rep = rep;
     c->colour = rep ? c->ws + ocol : nullptr;
-    c->normals = rep ? c->ws + onrm : nullptr;
+    c->rep_f = rep ? c->ws + onrm : nullptr;
   }
   return off;
 }

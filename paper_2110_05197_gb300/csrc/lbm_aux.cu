@@ -48,7 +48,7 @@ struct AuxParams {
   double nu_r, nu_b;
   double G, rho0, irho0; // SC two-component: G = G_eff; irho0 = 1 / rho0
   double body[3];
-  int forced;            // body is not 0
+  int forced;            // there may be a force: body is not 0, or repulsion
   double umax, neg_tol;
   double Ga[2], Gr[2];   // multirange SC self-couplings
   int px;                // row pitch and size of the stored arrays
@@ -80,7 +80,7 @@ AuxParams aux_params(const lbm_ctx* c) {
   a.rho0 = q.rho0_psi;
   a.irho0 = 1.0 / q.rho0_psi;
   for (int d = 0; d < 3; d++) a.body[d] = q.body_force[d];
-  a.forced = a.body[0] != 0 || a.body[1] != 0 || a.body[2] != 0;
+  a.forced = c->rep || a.body[0] != 0 || a.body[1] != 0 || a.body[2] != 0;
   a.umax = q.umax_unstable > 0 ? q.umax_unstable : 0.5;
   double scale = 1.0;
   if (q.model == LBM_MODEL_CG) scale = fmax(scale, fmax(q.rho_r0, q.rho_b0));
@@ -484,7 +484,7 @@ __device__ __forceinline__ void diag_finish(Acc& acc, double* __restrict__ parti
 // summation), psi of Eq. pseudopotential (SC multiphase, FP64), the momentum
 // j = sum_k sum_i c_i f^k_i into jm [3][N] (FP64), and for the multirange model the
 // pseudopotentials Psi_s of both species in the step's compute type into mrpsi [2][N].
-// FUSED (no force that depends on other nodes): the velocity and the totals as well, so that
+// FUSED (no stencil: colour gradient; rep, if not null: the repulsion force): the velocity and the totals as well, so that
 // neither the densities nor the momentum are read again.
 // rb may be null with one component.  `pitch`/`rows`: stored rows of `row` nodes, `pitch`
 // apart (one row of N nodes where they are dense); vld: pairs of stored nodes are aligned;
@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(kDiagThreads, 2) densities_kernel(
     const S* __restrict__ f0, const S* __restrict__ f1, const RT* __restrict__ r0, const RT* __restrict__ r1,
     lbm_diag* __restrict__ d, int cur, double* __restrict__ rr, double* __restrict__ rb, double* __restrict__ psi,
     double* __restrict__ jm, step_t<S>* __restrict__ mrpsi, const uint8_t* __restrict__ solid,
-    double* __restrict__ partials, AuxParams a, unsigned row, unsigned pitch, unsigned rows, int vld, int vst) {
+    double* __restrict__ partials, const step_t<S>* __restrict__ rep, AuxParams a, unsigned row, unsigned pitch, unsigned rows, int vld, int vst) {
   using C = step_t<S>;
   using V = typename Lanes<C>::V;
   constexpr int W = Lanes<C>::W, K = MODEL == LBM_MODEL_SC_MP ? 1 : 2;
@@ -569,9 +569,11 @@ __global__ void __launch_bounds__(kDiagThreads, 2) densities_kernel(
       for (int t = 0; t < 3; t++) out[2 + t][l] = jj[t];
       if (l && !two) break;
       if constexpr (FUSED) {
-        const double F[3] = {a.body[0], a.body[1], a.body[2]};
+        double F[3] = {a.body[0], a.body[1], a.body[2]};
         double u[3];
         const bool wall = solid && solid[n + l];
+        if (rep)
+          for (int t = 0; t < 3; t++) F[t] += widen(rep[t * a.n + n + l]);
         if (a.forced)
           diag_node<SUMS>(wall, out[0][l], out[1][l], jj, F, u, acc);
         else
@@ -667,14 +669,12 @@ __device__ __forceinline__ void sc_force(const double* __restrict__ rr, const do
 // FP64 issue bounds it (2 operations per clock and SM): every factor common to a stencil is
 // applied once to its sum.  128^3 SC multiphase 339 -> 183 us, two components 442 ->
 // 290 us.
-template <class L, class C, int MODEL, bool WALLS, bool SUMS>
+template <class L, int MODEL, bool WALLS, bool SUMS>
 __global__ void __launch_bounds__(kDiagThreads) diag_kernel(const double* __restrict__ rr,
                                                             const double* __restrict__ rb,
                                                             const double* __restrict__ psi,
                                                             const double* jm, const uint8_t* __restrict__ solid,
                                                             double* uo, double* __restrict__ partials, AuxParams a,
-                                                            const C* __restrict__ colour,
-                                                            const C* __restrict__ normals, RepParams rp,
                                                             lbm_diag* __restrict__ d, int cur) {
   Acc acc;
   acc_init(acc);
@@ -687,13 +687,7 @@ __global__ void __launch_bounds__(kDiagThreads) diag_kernel(const double* __rest
     if (!wall) {
       int x, y, z;
       node_xyz(n, a, x, y, z);
-      if constexpr (MODEL == LBM_MODEL_CG) {  // repulsion
-        C Fr[3];
-        rep_force<L, C>(normals, colour, WALLS ? solid : nullptr, x, y, z, rp, Fr);  // the step's own precision
-        for (int t = 0; t < 3; t++) F[t] += widen(Fr[t]);
-      } else {
-        sc_force<L, MODEL, WALLS>(rr, rb, psi, solid, r, b, n, x, y, z, a, F);
-      }
+      sc_force<L, MODEL, WALLS>(rr, rb, psi, solid, r, b, n, x, y, z, a, F);
     }
     double u[3];
     diag_node<SUMS>(wall, r, b, j, F, u, acc);
@@ -909,7 +903,8 @@ cudaError_t densities_t(lbm_ctx* c, const AuxParams& a, double* rr, double* rb, 
   const uint8_t* solid = c->has_walls ? c->solid : nullptr;
   densities_kernel<L, S, RT, MODEL, FUSED, SUMS><<<blocks, threads, 0, c->stream>>>(
       static_cast<const S*>(c->f[0]), static_cast<const S*>(c->f[1]), static_cast<const RT*>(c->r[0]),
-      static_cast<const RT*>(c->r[1]), c->diag, c->cur, rr, rb, psi, jm, mrpsi, solid, c->partials, a, (unsigned)row,
+      static_cast<const RT*>(c->r[1]), c->diag, c->cur, rr, rb, psi, jm, mrpsi, solid, c->partials,
+      c->rep ? static_cast<const C*>(c->rep_f) : nullptr, a, (unsigned)row,
       (unsigned)pitch, (unsigned)rows, vld, vst);
   c->launches += 1;
   return cudaGetLastError();
@@ -924,8 +919,13 @@ cudaError_t diag_t(lbm_ctx* c, double* rr, double* rb, double* uo) {
   double* jm = c->stage + 2 * c->N;   // momentum, then (if requested here) the velocity
   double* psi = c->stage + 5 * c->N;  // SC multiphase psi (FP64), or the multirange Psi_s
   const uint8_t* solid = c->has_walls ? c->solid : nullptr;
-  if constexpr (MODEL == LBM_MODEL_CG)
-    if (!c->rep) return densities_t<L, S, RT, MODEL, true, SUMS>(c, a, rr, rb, psi, uo);
+  if constexpr (MODEL == LBM_MODEL_CG) {
+    if (c->rep) {
+      cudaError_t e = launch_rep_prepass_t<L, C, S, RT>(c, c->cur);
+      if (e != cudaSuccess) return e;
+    }
+    return densities_t<L, S, RT, MODEL, true, SUMS>(c, a, rr, rb, psi, uo);
+  } else {
   cudaError_t e = densities_t<L, S, RT, MODEL, false, false>(c, a, rr, rb, psi, jm);
   if (e != cudaSuccess) return e;
   if constexpr (MODEL == LBM_MODEL_SC_MR) {
@@ -935,21 +935,14 @@ cudaError_t diag_t(lbm_ctx* c, double* rr, double* rb, double* uo) {
     kern<<<(int)std::min<long long>(units, c->nblk_diag), kDiagThreads, 0, c->stream>>>(
         rr, rb, reinterpret_cast<const C*>(psi), jm, solid, uo, c->partials, a, c->diag, c->cur);
   } else {
-    if (MODEL == LBM_MODEL_CG) {
-      e = launch_rep_prepass_t<L, C, S, RT>(c, c->cur);
-      if (e != cudaSuccess) return e;
-    }
-    // the SC forces do not depend on the compute type
-    using CK = typename std::conditional<MODEL == LBM_MODEL_CG, C, float>::type;
-    auto kern = solid ? diag_kernel<L, CK, MODEL, true, SUMS> : diag_kernel<L, CK, MODEL, false, SUMS>;
+    auto kern = solid ? diag_kernel<L, MODEL, true, SUMS> : diag_kernel<L, MODEL, false, SUMS>;
     const int threads = diag_threads(c, c->N);
     const int blocks = (int)std::min<long long>((c->N + threads - 1) / threads, c->nblk_diag);
-    kern<<<blocks, threads, 0, c->stream>>>(rr, rb, psi, jm, solid, uo, c->partials, a,
-                                                       static_cast<const CK*>(c->colour),
-                                                       static_cast<const CK*>(c->normals), rep_params(c), c->diag, c->cur);
+    kern<<<blocks, threads, 0, c->stream>>>(rr, rb, psi, jm, solid, uo, c->partials, a, c->diag, c->cur);
   }
   c->launches += 1;
   return cudaGetLastError();
+  }
 }
 
 // Dispatch on (lattice, storage precision) to an operation templated on <L, S, RT>.

@@ -61,21 +61,20 @@ size_t batch_ws_bytes(int max_jobs, int max_units) {
 template <class T, class S, class RT, bool WALLS>
 __device__ __forceinline__ void batch_march_w(const BatchJob<T, S, RT>& job, const StepArrays<S, RT>& a,
                                               const Segment& sg, unsigned char* smem) {
-  const RepParams rp{};
   if (job.lattice == LBM_D3Q19) {
     if (job.model == LBM_MODEL_CG)
-      march_segment<D3Q19, T, S, RT, kCG, WALLS, false, int>(a, job.p, nullptr, nullptr, rp, sg, smem);
+      march_segment<D3Q19, T, S, RT, kCG, WALLS, false, int>(a, job.p, nullptr, sg, smem);
     else if (job.model == LBM_MODEL_SC_MP)
-      march_segment<D3Q19, T, S, RT, kSCMP, WALLS, false, int>(a, job.p, nullptr, nullptr, rp, sg, smem);
+      march_segment<D3Q19, T, S, RT, kSCMP, WALLS, false, int>(a, job.p, nullptr, sg, smem);
     else
-      march_segment<D3Q19, T, S, RT, kSC2C, WALLS, false, int>(a, job.p, nullptr, nullptr, rp, sg, smem);
+      march_segment<D3Q19, T, S, RT, kSC2C, WALLS, false, int>(a, job.p, nullptr, sg, smem);
   } else {
     if (job.model == LBM_MODEL_CG)
-      march_segment<D2Q9, T, S, RT, kCG, WALLS, false, int>(a, job.p, nullptr, nullptr, rp, sg, smem);
+      march_segment<D2Q9, T, S, RT, kCG, WALLS, false, int>(a, job.p, nullptr, sg, smem);
     else if (job.model == LBM_MODEL_SC_MP)
-      march_segment<D2Q9, T, S, RT, kSCMP, WALLS, false, int>(a, job.p, nullptr, nullptr, rp, sg, smem);
+      march_segment<D2Q9, T, S, RT, kSCMP, WALLS, false, int>(a, job.p, nullptr, sg, smem);
     else
-      march_segment<D2Q9, T, S, RT, kSC2C, WALLS, false, int>(a, job.p, nullptr, nullptr, rp, sg, smem);
+      march_segment<D2Q9, T, S, RT, kSC2C, WALLS, false, int>(a, job.p, nullptr, sg, smem);
   }
 }
 

@@ -59,7 +59,7 @@ struct lbm_ctx {
   int occ_tx, occ_ty, occ_blocks;
   bool rep;              // CG repulsion force enabled (rep_pi != 0)
   void* colour;          // [N] rho^N (step compute type), repulsion pre-pass
-  void* normals;         // [3][N] unit colour gradients, repulsion pre-pass
+  void* rep_f;           // [3][N] repulsion force, pre-pass
   bool tma_ok;           // tensor maps built: the TMA-staged kernels can run this lattice
   lbm::TmaMaps tma[2];   // maps for reading buffer pair 0 / 1
 };
@@ -90,7 +90,7 @@ bool build_tma_maps(lbm_ctx* c);
 
 // Whether a lattice is stored for the pair kernel (lbm_step_pair.cuh): D3Q19, 32- or 16-bit
 // storage, two buffers, at most kPairMaxCluster tiles of 32 columns.  (The repulsion force
-// runs elsewhere, on the same storage.)
+// between walls runs elsewhere, on the same storage.)
 inline bool pair_lattice(const lbm_params& p) {
   return p.lattice == LBM_D3Q19 && p.precision != LBM_FP64 && p.streaming == LBM_STREAM_AB &&
          p.model != LBM_MODEL_SC_MR && p.nx <= 32 * kPairMaxCluster;
@@ -116,8 +116,6 @@ cudaError_t launch_aa_gather_plane(lbm_ctx* c, void* out, int k, int i);
 // left out), velocity into u_out unless that is null, the blow-up status and, if asked for,
 // the totals into the diagnostics record.
 cudaError_t launch_diagnostics(lbm_ctx* c, double* rho_r, double* rho_b, double* u_out, bool totals);
-// Repulsion pre-pass (colour and normal fields) of the current state, for the diagnostics.
-cudaError_t launch_rep_prepass(lbm_ctx* c);
 
 // Rest-state equilibrium weights per component and group: Eq. phi with alpha_k for CG
 // (alpha_R from Eq. gamma), the lattice weights w for SC.

@@ -34,6 +34,41 @@ __global__ void colour_kernel(const S* __restrict__ f, const RT* __restrict__ r,
   }
 }
 
+// The same on two nodes a thread (FP32 arithmetic, dense layout of the two-buffer scheme):
+// rows of `row` nodes, `pitch` apart, pairs of stored elements aligned.  256^3 FP16: 323 us
+// one node at a time, 224 (206 us are its bytes).
+template <class L, class S>
+__global__ void __launch_bounds__(256) colour2_kernel(const S* __restrict__ f, const float* __restrict__ r,
+                                                      float* __restrict__ colour, unsigned row, unsigned pitch,
+                                                      unsigned rows, RepParams a, long long ns) {
+  using U = typename std::conditional<sizeof(S) == 4, uint2, unsigned>::type;
+  const unsigned per = (row + 1) / 2, total = per * rows;
+  for (unsigned m = blockIdx.x * blockDim.x + threadIdx.x; m < total; m += gridDim.x * blockDim.x) {
+    const unsigned y = m / per, x = 2 * (m - y * per), st = y * pitch + x;
+    F2 rho[2];
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+      F2 g[L::Q];
+#pragma unroll
+      for (int i = 0; i < L::Q; i++) {
+        S e[2];
+        *reinterpret_cast<U*>(e) = *reinterpret_cast<const U*>(f + (k * L::Q + i) * ns + st);
+        g[i].set(0, ld_s<S, float>(e[0]));
+        g[i].set(1, ld_s<S, float>(e[1]));
+      }
+      rho[k] = comp_state2<L>(g, F2(*reinterpret_cast<const float2*>(r + k * ns + st))).q;
+    }
+#pragma unroll
+    for (int j = 0; j < 2; j++) {
+      float s0 = rho[0][j], s1 = rho[1][j];
+      if (a.color_norm) {
+        s0 = s0 * float(a.inv_rho_r0);
+        s1 = s1 * float(a.inv_rho_b0);
+      }
+      if (x + j < row) colour[y * row + x + j] = (s0 - s1) / (s0 + s1);
+    }
+  }
+}
 
 inline RepParams rep_params(const lbm_ctx* c) {
   RepParams a{};
@@ -51,21 +86,35 @@ inline RepParams rep_params(const lbm_ctx* c) {
   return a;
 }
 
-// Colour and normal fields of the current state (repulsion pre-pass).
+// Repulsion force of the current state into c->rep_f.
 template <class L, class T, class S, class RT>
 cudaError_t launch_rep_prepass_t(lbm_ctx* c, int buf) {
   const RepParams a = rep_params(c);
   const int grid = (int)std::min<long long>((c->N + 255) / 256, 8192);
-  colour_kernel<L, T, S, RT><<<grid, 256, 0, c->stream>>>(static_cast<const S*>(c->f[buf]),
-                                                           static_cast<const RT*>(c->r[buf]),
-                                                           static_cast<T*>(c->colour), a, c->aa ? (buf & 1) : 0,
-                                                           c->px, c->NS);
-  if (3 * c->N < (1LL << 31))  // 32-bit indices: the normals array holds 3 N values
-    normals_kernel<L, T, int><<<grid, 256, 0, c->stream>>>(
-        static_cast<const T*>(c->colour), c->has_walls ? c->solid : nullptr, static_cast<T*>(c->normals), a);
-  else
-    normals_kernel<L, T, long long><<<grid, 256, 0, c->stream>>>(
-        static_cast<const T*>(c->colour), c->has_walls ? c->solid : nullptr, static_cast<T*>(c->normals), a);
+  const S* f = static_cast<const S*>(c->f[buf]);
+  const RT* r = static_cast<const RT*>(c->r[buf]);
+  T* colour = static_cast<T*>(c->colour);
+  bool two = false;
+  if constexpr (sizeof(T) == 4) {
+    const bool dense = c->px == c->p.nx;
+    const long long row = dense ? c->N : c->p.nx, pitch = dense ? c->N : c->px, rows = c->N / row;
+    two = !c->aa && pitch % 2 == 0 && c->NS % 2 == 0 && c->NS < (1LL << 32);
+    if (two)
+      colour2_kernel<L, S><<<(grid + 1) / 2, 256, 0, c->stream>>>(f, r, colour, (unsigned)row, (unsigned)pitch,
+                                                                  (unsigned)rows, a, c->NS);
+  }
+  if (!two)
+    colour_kernel<L, T, S, RT><<<grid, 256, 0, c->stream>>>(f, r, colour, a, c->aa ? (buf & 1) : 0, c->px, c->NS);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  // planes per block: long runs share their halo planes, short ones keep the SMs busy
+  const long long tiles = (long long)((c->p.nx + kRepTX - 1) / kRepTX) * ((c->p.ny + kRepTY - 1) / kRepTY);
+  int chunk = 16;
+  while (chunk > 1 && tiles * ((c->p.nz + chunk - 1) / chunk) < 8LL * c->nsm) chunk /= 2;
+  const long long blocks = tiles * ((c->p.nz + chunk - 1) / chunk);
+  if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
+  auto kern = c->has_walls ? rep_force_kernel<L, T, true> : rep_force_kernel<L, T, false>;
+  kern<<<(int)blocks, kRepThreads, 0, c->stream>>>(colour, c->solid, static_cast<T*>(c->rep_f), chunk, a);
   c->launches += 2;
   return cudaGetLastError();
 }
@@ -120,10 +169,10 @@ cudaError_t launch_tma_t(lbm_ctx* c) {
 
 // Pair kernel (lbm_step_pair.cuh): clusters of nx / 32 blocks, each cluster one run of
 // (tile row, plane) pairs; TY rows per tile, MB blocks per SM.
-template <class L, class T, class S, class RT, int MODEL, int FORM, int TY, int MB>
+template <class L, class T, class S, class RT, int MODEL, int FORM, int TY, int MB, bool REP = false>
 cudaError_t launch_pair_tile(lbm_ctx* c) {
   constexpr size_t smem = pair_smem_bytes<L, S, RT, MODEL, TY>(pair_raw<L, S, RT, MODEL, TY, MB>());
-  auto kern = step_kernel_pair<L, T, S, RT, MODEL, FORM, TY, MB>;
+  auto kern = step_kernel_pair<L, T, S, RT, MODEL, FORM, TY, MB, REP>;
   static bool attr_set = false;
   if (!attr_set) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -163,7 +212,7 @@ cudaError_t launch_pair_tile(lbm_ctx* c) {
   for (int a = 0; a < c->K * c->Q; a++) out.f[a] = static_cast<S*>(c->f[c->cur ^ 1]) + a * c->NS;
   for (int k = 0; k < c->K; k++) out.r[k] = static_cast<RT*>(c->r[c->cur ^ 1]) + k * c->NS;
   return cudaLaunchKernelEx(&cfg, kern, c->tma[c->cur], out, static_cast<const uint8_t*>(c->near_wall),
-                            &c->diag->status, sp);
+                            static_cast<const T*>(c->rep_f), &c->diag->status, sp);
 }
 
 // Tile of the pair kernel.  CG keeps a plane's sums in registers (242 of them), two-component
@@ -172,10 +221,16 @@ cudaError_t launch_pair_tile(lbm_ctx* c) {
 // (128^3: 68 us against 73), unless 16 rows do not divide ny or there are fewer such tiles
 // than blocks to hold them (32^3: 10.4 us against 8.8); in 16-bit storage, whose plane
 // buffers are half as large, as four blocks of 8 rows (57.6 against 59.8 us).
-template <class L, class T, class S, class RT, int MODEL, bool WALLS>
+template <class L, class T, class S, class RT, int MODEL, bool WALLS, bool REP>
 cudaError_t launch_pair_t(lbm_ctx* c) {
   constexpr int MB = MODEL != kSCMP ? 2 : sizeof(S) == 4 ? 3 : 4;
-  if constexpr (WALLS) {
+  if constexpr (REP) {
+    static_assert(!WALLS, "the repulsion force between walls runs on the generic kernel");
+    cudaError_t e = launch_rep_prepass_t<L, T, S, RT>(c, c->cur);
+    if (e != cudaSuccess) return e;
+    if (c->p.nx % kPairTX != 0 || c->p.ny % 8 != 0) return launch_pair_tile<L, T, S, RT, MODEL, kRagged, 8, MB, true>(c);
+    return launch_pair_tile<L, T, S, RT, MODEL, kFull, 8, MB, true>(c);
+  } else if constexpr (WALLS) {
     cudaError_t e = launch_pair_tile<L, T, S, RT, MODEL, kWalls, 8, MB>(c);
     if (e != cudaSuccess) return e;
     c->launches += 1;
@@ -252,12 +307,10 @@ cudaError_t launch_fp_i(lbm_ctx* c) {
     tp.ncol = tp.ncx * ((c->p.ny + kFpTY - 1) / kFpTY);
     persistent_plan(tp, c->nsm * occ);
     kern<<<tp.nblk, kFpTX * kFpTY, smem, c->stream>>>(fin, fout, rin, rout, fld, c->solid, &c->diag->status, tp,
-                                                      static_cast<const T*>(c->colour),
-                                                      static_cast<const T*>(c->normals), rep_params(c), mode);
+                                                      static_cast<const T*>(c->rep_f), mode);
   } else {
     fp_step_kernel<L, T, S, RT, MODEL, WALLS, REP, I><<<grid, 256, 0, c->stream>>>(
-        fin, fout, rin, rout, fld, c->solid, &c->diag->status, sp, static_cast<const T*>(c->colour),
-        static_cast<const T*>(c->normals), rep_params(c), mode);
+        fin, fout, rin, rout, fld, c->solid, &c->diag->status, sp, static_cast<const T*>(c->rep_f), mode);
   }
   return cudaGetLastError();
 }
@@ -305,8 +358,7 @@ cudaError_t launch_generic_t(lbm_ctx* c) {
   const RT* rin = static_cast<const RT*>(c->r[c->cur]);
   RT* rout = static_cast<RT*>(c->r[c->cur ^ 1]);
   step_kernel<L, T, S, RT, MODEL, WALLS, REP, I><<<grid, block, smem, c->stream>>>(
-      fin, fout, rin, rout, c->solid, &c->diag->status, sp, static_cast<const T*>(c->colour),
-      static_cast<const T*>(c->normals), rep_params(c));
+      fin, fout, rin, rout, c->solid, &c->diag->status, sp, static_cast<const T*>(c->rep_f));
   return cudaGetLastError();
 }
 
@@ -317,8 +369,8 @@ cudaError_t launch_step_t(lbm_ctx* c) {
   } else {
   if (c->aa) return launch_fp_t<L, T, S, RT, MODEL, WALLS, REP>(c);
   // the pair kernel, whatever the tiling
-  if constexpr (L::D == 3 && sizeof(T) == 4 && !REP)
-    if (pair_steps(c)) return launch_pair_t<L, T, S, RT, MODEL, WALLS>(c);
+  if constexpr (L::D == 3 && sizeof(T) == 4 && !(REP && WALLS))
+    if (pair_steps(c)) return launch_pair_t<L, T, S, RT, MODEL, WALLS, REP>(c);
   if (c->tx * c->ty > 256) {
     // the 512-node tilings run as 32 x 8 persistent tiles
     const int tx = c->tx, ty = c->ty, tz = c->tz;

@@ -561,13 +561,12 @@ struct StepArrays {
 // March one work unit (column sg.col, planes [sg.z0, sg.z1)) of a lattice through a full
 // step with the block's TX x TY threads; smem_raw holds step_smem_bytes() bytes.  Ends with
 // a block barrier, so the caller may reuse shared memory right away.
-// REP (CG only): add the repulsion force of Eq. repForce from the pre-pass fields
-// colour / normals (lbm_rep.cuh).  I: the integer type of node and array indices, int
+// REP (CG only): add the repulsion force of Eq. repForce from the pre-pass field rep [3][n]
+// (lbm_rep.cuh).  I: the integer type of node and array indices, int
 // when K * Q * ns < 2^31 (the launcher's choice), else long long.
 template <class L, class T, class S, class RT, int MODEL, bool WALLS, bool REP, class I = long long>
 __device__ __forceinline__ void march_segment(const StepArrays<S, RT>& a, const StepParams<T>& p,
-                                              const T* __restrict__ colour, const T* __restrict__ normals,
-                                              const RepParams& rp, const Segment& sg,
+                                              const T* __restrict__ rep, const Segment& sg,
                                               unsigned char* __restrict__ smem_raw) {
   constexpr int Q = L::Q;
   constexpr int K = ModelTraits<MODEL>::K, NF = ModelTraits<MODEL>::NF;
@@ -652,7 +651,11 @@ __device__ __forceinline__ void march_segment(const StepArrays<S, RT>& a, const 
     };
     if constexpr (MODEL == kCG) {
       T Fx[3] = {T(0), T(0), T(0)};
-      if constexpr (REP) rep_force<L, T, I>(normals, colour, WALLS ? solid : nullptr, gx, gy, z, rp, Fx);
+      if constexpr (REP) {
+        const I nd = gx + I(p.nx) * (gy + I(p.ny) * z);
+#pragma unroll
+        for (int a = 0; a < 3; a++) Fx[a] = rep[I(a) * I(p.n) + nd];
+      }
       cg_collide<L, T>(p, g, cs[0], cs[1], nbr, Fx);
     } else if constexpr (MODEL == kSCMP) {
       scmp_collide<L, T>(p, g, cs[0], nbr);
@@ -719,13 +722,13 @@ template <class L, class T, class S, class RT, int MODEL, bool WALLS, bool REP, 
 __global__ void __launch_bounds__(256, min_blocks<T>()) step_kernel(
     const S* __restrict__ fin, S* __restrict__ fout, const RT* __restrict__ rin, RT* __restrict__ rout,
     const uint8_t* __restrict__ solid, const int* __restrict__ status, const __grid_constant__ StepParams<T> p,
-    const T* __restrict__ colour, const T* __restrict__ normals, const __grid_constant__ RepParams rp) {
+    const T* __restrict__ rep) {
   if (status != nullptr && *status != 0) return;  // blown-up state: stop stepping
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const StepArrays<S, RT> a{fin, fout, rin, rout, solid};
   WorkRange work(blockIdx.x, p.nblk, p.ncol, p.nz, p.nchunks);
   Segment sg;
-  while (work.pop(sg)) march_segment<L, T, S, RT, MODEL, WALLS, REP, I>(a, p, colour, normals, rp, sg, smem_raw);
+  while (work.pop(sg)) march_segment<L, T, S, RT, MODEL, WALLS, REP, I>(a, p, rep, sg, smem_raw);
 }
 
 }  // namespace lbm

@@ -101,8 +101,7 @@ template <class L, class T, class S, class RT, int MODEL, bool WALLS, bool REP, 
 __global__ void __launch_bounds__(256, min_blocks<T>())
     fp_step_kernel(const S* fin, S* fout, const RT* rin, RT* rout, const T* __restrict__ fld,
                    const uint8_t* __restrict__ solid, const int* __restrict__ status,
-                   const __grid_constant__ StepParams<T> p, const T* __restrict__ colour,
-                   const T* __restrict__ normals, const __grid_constant__ RepParams rp, int mode) {
+                   const __grid_constant__ StepParams<T> p, const T* __restrict__ rep, int mode) {
   if (*status != 0) return;
   const bool inplace = mode != 0, odd = mode == 2;
   constexpr int Q = L::Q, K = ModelTraits<MODEL>::K, NF = ModelTraits<MODEL>::NF;
@@ -140,7 +139,8 @@ __global__ void __launch_bounds__(256, min_blocks<T>())
     };
     if constexpr (MODEL == kCG) {
       T Fx[3] = {T(0), T(0), T(0)};
-      if constexpr (REP) rep_force<L, T, I>(normals, colour, WALLS ? solid : nullptr, x, y, z, rp, Fx);
+      if constexpr (REP)
+        for (int a = 0; a < 3; a++) Fx[a] = rep[I(a) * N + n];
       cg_collide<L, T>(p, g, cs[0], cs[1], nbr, Fx);
     } else if constexpr (MODEL == kSCMR) {
       auto far = [&](int fi, int dx, int dy, int dz) -> T {
@@ -197,8 +197,7 @@ template <class L, class T, class S, class RT, int MODEL, bool WALLS, bool REP, 
 __global__ void __launch_bounds__(kFpTX * kFpTY, min_blocks<T>())
     fpt_step_kernel(const S* fin, S* fout, const RT* rin, RT* rout, const T* __restrict__ fld,
                     const uint8_t* __restrict__ solid, const int* __restrict__ status,
-                    const __grid_constant__ StepParams<T> p, const T* __restrict__ colour,
-                    const T* __restrict__ normals, const __grid_constant__ RepParams rp, int mode) {
+                    const __grid_constant__ StepParams<T> p, const T* __restrict__ rep, int mode) {
   if (*status != 0) return;
   static_assert(L::D == 3, "plane marching");
   constexpr int TX = kFpTX, TY = kFpTY;
@@ -264,7 +263,8 @@ __global__ void __launch_bounds__(kFpTX * kFpTY, min_blocks<T>())
         auto nbr = [&](int fi, int i) -> T { return at(fi, cx<L>(i), cy<L>(i), cz<L>(i)); };
         if constexpr (MODEL == kCG) {
           T Fx[3] = {T(0), T(0), T(0)};
-          if constexpr (REP) rep_force<L, T, I>(normals, colour, WALLS ? solid : nullptr, x, y, z, rp, Fx);
+          if constexpr (REP)
+            for (int a = 0; a < 3; a++) Fx[a] = rep[I(a) * N + n];
           cg_collide<L, T>(p, g, cs[0], cs[1], nbr, Fx);
         } else if constexpr (MODEL == kSCMR) {
           scmr_collide<L, T>(p, g, cs[0], cs[1], nbr, at);

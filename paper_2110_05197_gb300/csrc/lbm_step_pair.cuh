@@ -114,9 +114,11 @@ struct PairSum {
 // c.grad rho) + K3 (c.grad rho^N)^2 and O = K4 cu, whose group constants K hold the relaxed
 // equilibrium (Eqs. BGK, equiliCG), the perturbation (Eq. perturbationOp) and the change of
 // reference, with S0, S1 the Guo source (Eq. source) of a body force.
-template <class L, class NB, class READY, class EMIT>
+// REP: the nodes' repulsion forces fr come on top of the body force.
+template <class L, bool REP, class NB, class READY, class EMIT>
 __device__ __forceinline__ void cg_collide_pair(const StepParams<float>& p, const F2 (&t)[L::Q], const Comp2& cr,
-                                                const Comp2& cb, const NB& nb, const READY& ready, const EMIT& emit) {
+                                                const Comp2& cb, const F2 (&fr)[3], const NB& nb, const READY& ready,
+                                                const EMIT& emit) {
   const F2 qR = cr.q, qB = cb.q;
   PairSum<L> sj;
 #pragma unroll
@@ -125,13 +127,19 @@ __device__ __forceinline__ void cg_collide_pair(const StepParams<float>& p, cons
   const F2 rho = qR + qB;
   const F2 inv = each(rho, rcp);
   F2 u[3], F[3];
-  const bool forced = p.has_body;
+  bool forced = p.has_body;
+  if constexpr (REP) {  // away from interfaces every force of the warp is 0
+    const bool any = fr[0][0] != 0.f || fr[0][1] != 0.f || fr[1][0] != 0.f || fr[1][1] != 0.f || fr[2][0] != 0.f ||
+                     fr[2][1] != 0.f;
+    forced = forced || __any_sync(0xffffffffu, any);
+  }
 #pragma unroll
   for (int k = 0; k < 3; k++) {
     F2 jm = k < L::D ? sj.ax[k] + sj.dg[k] : F2(0.f);
-    if (forced) jm = jm + F2(0.5f * p.body[k]);
-    u[k] = jm * inv;
     F[k] = F2(p.body[k]);
+    if constexpr (REP) F[k] = F[k] + fr[k];
+    if (forced) jm = REP ? fma(F2(0.5f), F[k], jm) : jm + F2(0.5f * p.body[k]);
+    u[k] = jm * inv;
   }
   const F2 sv = fma(qR, F2(p.inv_nu_r), qB * F2(p.inv_nu_b));
   const F2 nubar = rho * each(sv, rcp);
@@ -501,13 +509,14 @@ enum PairForm : int { kFull = 0, kRagged = 1, kWalls = 2 };
 // p.nblk clusters * C blocks of 16 TY threads, MB blocks per SM; p.ncol = ceil(ny / TY) tile
 // rows.  Rows are p.px nodes apart (a multiple of 16 bytes, which a tensor map needs), the
 // last tile of a row or column may be partial.  Every index within an array fits 31 bits.
+// REP (colour gradient): the repulsion force rep [3][n] of lbm_rep.cuh is added.
 // With walls (kWalls) the nodes beside one are left to wall_step_kernel, except for their
 // reference densities, which it reads.
-template <class L, class T, class S, class RT, int MODEL, int FORM, int TY, int MB>
+template <class L, class T, class S, class RT, int MODEL, int FORM, int TY, int MB, bool REP = false>
 __global__ void __launch_bounds__(16 * TY, MB)
     step_kernel_pair(const __grid_constant__ TmaMaps maps,
                      const __grid_constant__ OutArrays<S, RT, ModelTraits<MODEL>::K * L::Q, ModelTraits<MODEL>::K> out,
-                     const uint8_t* __restrict__ near_wall, int* __restrict__ status,
+                     const uint8_t* __restrict__ near_wall, const T* __restrict__ rep, int* __restrict__ status,
                      const __grid_constant__ StepParams<T> p) {
   static_assert(sizeof(T) == 4 && sizeof(RT) == 4, "fields are exchanged as 32-bit words");
   static_assert(TY == 8 || TY == 16, "tile rows with a tensor map");
@@ -672,6 +681,18 @@ __global__ void __launch_bounds__(16 * TY, MB)
         stage_rows(0, TY + 1, 0, rows + 1, false, unused);
       }
     }
+    // repulsion forces of the nodes collided below, on their way during the barrier
+    [[maybe_unused]] F2 fr[3];
+    if constexpr (REP) {
+#pragma unroll
+      for (int k = 0; k < 3; k++)
+#pragma unroll
+        for (int j = 0; j < 2; j++) {
+          const bool own = prev_interior && (FULL || !(near[j] & kWallSelf));
+          const unsigned n = x0 + lane + p.nx * (prev_y0 + 2 * warp + j + p.ny * prev_z);
+          fr[k].set(j, own ? rep[k * p.n + n] : 0.f);
+        }
+    }
     __syncthreads();  // local fields of plane J complete; iteration J-1 retired
     issue_next();     // into this plane's buffer (EARLY), else into plane J-1's
     if (alive && (lane == 0 || lane == width - 1)) {
@@ -749,7 +770,7 @@ __global__ void __launch_bounds__(16 * TY, MB)
           push(0, 0, i, vR);
           push(1, 1, i, vB);
         };
-        cg_collide_pair<L>(p, hold, hcs[0], hcs[1], nb, ready, emit);
+        cg_collide_pair<L, REP>(p, hold, hcs[0], hcs[1], fr, nb, ready, emit);
       } else if constexpr (MODEL == kSC2C) {
         auto emit = [&](int k, int i, const F2& v) { push(k, k, i, v); };
         sc2c_collide_pair<L>(p, hold, hcs, nb, ready, emit);
