@@ -327,7 +327,31 @@ cudaError_t launch_fp_t(lbm_ctx* c) {
 // Generic plane-marching step (step_kernel) with index type I.
 template <class L, class T, class S, class RT, int MODEL, bool WALLS, bool REP, class I>
 cudaError_t launch_generic_t(lbm_ctx* c) {
-  const int tx = c->tx, ty = c->ty;
+  const int tx = c->tx;
+  int ty = c->ty, tz = c->tz;
+  // A lattice with fewer tiles than SMs is cut into smaller ones: the time is that of the
+  // fullest SM, whose tiles take a collision per node and a staging (about a quarter of one)
+  // per node and halo node.  2D 128^2 CG FP64 (32 x 8 tiles on 64 SMs): 31.8 us, as 32 x 4
+  // tiles on 128 19.5.
+  const long long tiles_x = (c->p.nx + tx - 1) / tx;
+  auto units = [&](int y, int z) {
+    return tiles_x * ((c->p.ny + y - 1) / y) * (z > 0 ? (c->p.nz + z - 1) / z : 1);
+  };
+  if (tz > 0 && units(ty, tz) < c->nsm) {
+    auto cost = [&](int y, int z) {
+      const long long rounds = (units(y, z) + c->nsm - 1) / c->nsm;
+      return double(rounds) * (double(tx) * y * z + 0.25 * (tx + 2) * (y + 2) * (L::D == 3 ? z + 2 : 1));
+    };
+    double best = cost(ty, tz);
+    const int y0 = ty, z0 = tz;
+    for (int z = z0; z >= 1; z /= 2)
+      for (int y = y0; y >= 1 && tx * y >= 64; y /= 2)
+        if (cost(y, z) < best) {
+          best = cost(y, z);
+          ty = y;
+          tz = z;
+        }
+  }
   const size_t smem = step_smem_bytes<L, T, MODEL, WALLS>(tx, ty);
   static size_t smem_set = 0;  // largest dynamic shared memory opted in so far
   if (smem > 48 * 1024 && smem > smem_set) {
@@ -338,7 +362,10 @@ cudaError_t launch_generic_t(lbm_ctx* c) {
   }
   dim3 block(tx, ty, 1);
   StepParams<T> sp = make_step_params<T>(c);
-  if (c->tz == 0) {
+  sp.ncol = (int)units(ty, 0);
+  sp.nchunks = tz > 0 ? (c->p.nz + tz - 1) / tz : 1;
+  sp.nblk = sp.ncol * sp.nchunks;
+  if (tz == 0) {
     const void* fn = reinterpret_cast<const void*>(step_kernel<L, T, S, RT, MODEL, WALLS, REP, I>);
     if (c->occ_fn != fn || c->occ_tx != tx || c->occ_ty != ty) {
       int nb = 0;
