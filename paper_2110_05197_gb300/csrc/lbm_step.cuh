@@ -718,11 +718,22 @@ __device__ __forceinline__ void march_segment(const StepArrays<S, RT>& a, const 
   }
 }
 
+// Steps of one lattice follow each other as programmatic dependent launches: the next step's
+// blocks are set up while this one's last blocks still run, and wait here, before they touch
+// global memory, until the step before has completed and its writes are visible.  Per step of
+// a run, plain launches -> these: 2D 256^2 SC FP32 6.0 -> 4.2 us, 32^3 CG FP32 12.2 -> 8.9, 2D
+// 128^2 CG FP64 19.5 -> 16.8, 128^3 SC FP32 68 -> 67.
+__device__ __forceinline__ void await_previous_step() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 template <class L, class T, class S, class RT, int MODEL, bool WALLS, bool REP, class I = long long>
 __global__ void __launch_bounds__(256, min_blocks<T>()) step_kernel(
     const S* __restrict__ fin, S* __restrict__ fout, const RT* __restrict__ rin, RT* __restrict__ rout,
     const uint8_t* __restrict__ solid, const int* __restrict__ status, const __grid_constant__ StepParams<T> p,
     const T* __restrict__ rep) {
+  await_previous_step();
   if (status != nullptr && *status != 0) return;  // blown-up state: stop stepping
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const StepArrays<S, RT> a{fin, fout, rin, rout, solid};

@@ -529,9 +529,6 @@ __global__ void __launch_bounds__(16 * TY, MB)
   constexpr int NV = PairTraits<MODEL>::NV, NH = PairTraits<MODEL>::NH;
   constexpr int EX = Lay::EX, NE = Lay::NE;
   constexpr int FS = kPairFields;
-  // A blown-up (or timed-out) state stops stepping; the cluster barriers are still passed.
-  const bool skip = *status != 0;
-
   extern __shared__ __align__(128) unsigned char smem[];
   uint64_t* raw_full = reinterpret_cast<uint64_t*>(smem);     // [RAW]
   uint64_t* fld_full = raw_full + RAW;                         // [FS]: the neighbours' columns
@@ -555,6 +552,9 @@ __global__ void __launch_bounds__(16 * TY, MB)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   cluster_sync_all();  // barriers of every block initialised before any remote store
+  await_previous_step();
+  // A blown-up (or timed-out) state stops stepping; the cluster barriers are still passed.
+  const bool skip = *status != 0;
   // copy destinations must be 128-byte aligned; a misaligned base stops the work (every
   // block of the cluster sees the same offset) but not the barriers
   const bool layout_ok = (smem_addr(bufs) & 127u) == 0;
