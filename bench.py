@@ -254,14 +254,10 @@ def serving_sweep(n_req: int, seed: int = 5):
     return out
 
 
-def kernel_label(model: str, precision: int, tiling) -> str:
-    """The step kernel a tiling runs on the 128^3 benchmark lattices: the pair kernel for the
-    tilings that name a TMA-staged kernel, the generic kernel otherwise."""
+def kernel_label(model: str, precision: int) -> str:
+    """The step kernel of the 128^3 benchmark lattices: the pair kernel, whatever the tiling."""
     elt = {1: "float", 2: "half", 3: "bf16"}[precision]
-    m = "CG" if model == "cg" else "SC-MP"
-    if (int(tiling[0]), int(tiling[1])) in ((32, 8), (32, 4), (64, 4), (32, 16), (64, 8)):
-        return f"step_kernel_pair<D3Q19,{elt},{m}>"
-    return f"step_kernel<D3Q19,{elt},{m}>"
+    return f"step_kernel_pair<D3Q19,{elt},{'CG' if model == 'cg' else 'SC-MP'}>"
 
 
 def storage16_steps(rr, rb, rho, dev, stream, steps: int = 20):
@@ -286,7 +282,7 @@ def storage16_steps(rr, rb, rho, dev, stream, steps: int = 20):
         ms = a.elapsed_time(b) / steps
         gbs = out["bytes_per_lu"][name] * N3 ** 3 / (ms / 1e3) / 1e9
         out[name] = {"step_ms": ms, "mlups": N3 ** 3 / (ms / 1e3) / 1e6, "achieved_gbs": gbs,
-                     "frac": gbs / peak, "tiling": list(best), "kernel": kernel_label(name, lbm.FP16, best),
+                     "frac": gbs / peak, "tiling": list(best), "kernel": kernel_label(name, lbm.FP16),
                      "status": lbm.status_string(lat.totals()[1])}
         lat.close()
     return out
@@ -501,8 +497,8 @@ def run_ours(args):
     cg_avg, sc_avg = float(np.mean(cg_ms)), float(np.mean(sc_ms))
     value = job_mlups(n, 2, K, ws, total_ms / 1e3)
     peak, peak_kind = hbm_peak()
-    cg_kernel = kernel_label("cg", lbm.FP32, tiling["cg"])
-    sc_kernel = kernel_label("sc", lbm.FP32, tiling["sc"])
+    cg_kernel = kernel_label("cg", lbm.FP32)
+    sc_kernel = kernel_label("sc", lbm.FP32)
     achieved = BYTES_PER_LU["cg"] * n / (cg_avg / 1e3) / 1e9
     tot_cg, rc_cg = cg.totals()
     tot_sc, rc_sc = sc.totals()

@@ -82,9 +82,8 @@ __device__ __forceinline__ void cp_async_arrive_noinc(uint64_t* bar) {
 // Bounded wait on an mbarrier phase (the copies complete on their own; the bound keeps a
 // lost completion from hanging the GPU).  After one plain test, each try_wait carries a
 // suspend-time hint, so a waiting warp sleeps until the phase completes (or the hint
-// elapses) instead of re-polling: the producer and staging warps of the cluster kernel
-// wait for most of each plane, and their polling took issue slots from the collision
-// warps (128^3 CG FP32 cluster kernel 183 -> 179 us, 16-bit CG 159 -> 154 us).  The wait
+// elapses) instead of re-polling: producer and staging warps wait for most of each plane,
+// and their polling takes issue slots from the collision warps (2% to 3% of a step).  The wait
 // gives up after kWaitNs of global time or kWaitLimit tries, whichever comes first.
 constexpr long long kWaitLimit = 1LL << 22;
 constexpr uint32_t kSuspendNs = 20000;
@@ -154,7 +153,7 @@ struct TmaLayout {
   static constexpr int HW = KQ + K;                  // halo words per side and row
   static constexpr int NH = 2 * EY * HW;             // halo words per plane
   static constexpr size_t BUF = (OFF_H + size_t(NH) * 4 + 127) & ~size_t(127);
-  static constexpr size_t BUF_MAIN = OFF_H;          // without the halo words (cluster kernel)
+  static constexpr size_t BUF_MAIN = OFF_H;          // without the halo words (pair kernel)
   static_assert(BUF % 128 == 0 && OFF_RM % 128 == 0, "tensor-copy destinations must be 128-byte aligned");
   // bytes the tensor copies of one plane deliver (the alignment padding is not written)
   static constexpr uint32_t TX_BYTES = uint32_t(EY) * (KQ * TX * sizeof(S) + K * TX * sizeof(RT));
