@@ -225,6 +225,9 @@ cudaError_t launch_pair_tile(lbm_ctx* c) {
     c->occ_blocks = ncl > 0 ? ncl : 1;
   }
   sp.nblk = (int)std::min<long long>(c->occ_blocks, (long long)sp.ncol * sp.nz);  // clusters
+  // a grid of at most one block per SM leaves room for the next step's blocks beside its own: they
+  // come before its last collision (32^3 CG FP32 9.3 -> 8.7 us)
+  sp.admit_early = sp.nblk * C <= c->nsm;
   // the step follows the step before as a programmatic dependent launch, but not between walls:
   // the waiting blocks of the next kernel then hold up the clusters (101 x 75 x 67: 66 -> 81 us)
   cfg.numAttrs = FORM == kWalls ? 1 : 2;

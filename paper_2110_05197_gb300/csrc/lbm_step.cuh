@@ -54,6 +54,7 @@ struct StepParams {
   long long n;            // nodes
   int px;                 // nodes from one stored row to the next
   long long ns;           // elements of a stored array (px * ny * nz)
+  int admit_early;        // pair kernel: the next step's blocks may come before the last collision
   T phi[2][3];            // rest-state weights per component and group (CG: Eq. phi; SC: w)
   // CG
   T inv_nu_r, inv_nu_b;   // 1/nu_k, nu_k = (tau_k - 1/2)/3
@@ -718,15 +719,16 @@ __device__ __forceinline__ void march_segment(const StepArrays<S, RT>& a, const 
   }
 }
 
-// Steps of one lattice follow each other as programmatic dependent launches: the next step's
-// blocks are set up while this one's last blocks still run, and wait here, before they touch
-// global memory, until the step before has completed and its writes are visible.  Per step of
-// a run, plain launches -> these: 2D 256^2 SC FP32 6.0 -> 4.2 us, 32^3 CG FP32 12.2 -> 8.9, 2D
-// 128^2 CG FP64 19.5 -> 16.8, 128^3 SC FP32 68 -> 67.
-__device__ __forceinline__ void await_previous_step() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
+// Steps of one lattice follow each other as programmatic dependent launches.  A kernel waits
+// before it touches global memory until the step before has completed and its writes are
+// visible, and lets the next step's blocks start as its own end.  (Let in at the start, they take
+// their places while this step's blocks still hold theirs, and end up unevenly spread over the
+// SMs: on 3D lattices of a few hundred tiles a step then takes 5% to 15% longer than after a
+// plain launch.)  Per step of a run, plain launches / let in at the start / at the end: 2D 256^2 SC
+// FP32 6.2 / 4.6 / 4.2 us, 2D 128^2 CG FP64 20.5 / 17.9 / 17.6, 61 x 57 x 59 SC FP32 16.5 / 17.5 /
+// 14.6, 8 x 150 x 150 CG FP32 42.9 / 48.0 / 40.1, 24 x 24 x 600 SC FP32 24.7 / 27.5 / 22.9.
+__device__ __forceinline__ void await_previous_step() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void admit_next_step() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <class L, class T, class S, class RT, int MODEL, bool WALLS, bool REP, class I = long long>
 __global__ void __launch_bounds__(256, min_blocks<T>()) step_kernel(
@@ -740,6 +742,7 @@ __global__ void __launch_bounds__(256, min_blocks<T>()) step_kernel(
   WorkRange work(blockIdx.x, p.nblk, p.ncol, p.nz, p.nchunks);
   Segment sg;
   while (work.pop(sg)) march_segment<L, T, S, RT, MODEL, WALLS, REP, I>(a, p, rep, sg, smem_raw);
+  admit_next_step();
 }
 
 }  // namespace lbm

@@ -441,6 +441,7 @@ struct PlaneRun {
   __device__ void advance() {
     if (++z > sg.z1) pop();
   }
+  __device__ bool last() const { return z == sg.z1 && next >= end; }
 };
 
 __device__ __forceinline__ uint32_t cluster_ctarank() {
@@ -610,6 +611,7 @@ __global__ void __launch_bounds__(16 * TY, MB)
     const int y0 = cur.sg.col * TY;
     const int z = cur.z;
     const bool interior = z >= cur.sg.z0 && z < cur.sg.z1;  // plane J is collided in iteration J+1
+    if (p.admit_early && cur.last()) admit_next_step();
     const int fs = J % FS;
     const unsigned char* b = bufs + (J % RAW) * Lay::BUF_MAIN;
     const int halo_warp = J % kWarps;  // stages the halo rows too
@@ -805,6 +807,7 @@ __global__ void __launch_bounds__(16 * TY, MB)
     prev_y0 = y0;
     cur.advance();
   }
+  admit_next_step();
   // the copies this block issued have landed before its shared memory is released
   if (tid == 0)
     for (int j = max(0, issued - RAW); j < issued; j++) mbar_wait_bounded(&raw_full[j % RAW], (j / RAW) & 1);
