@@ -111,8 +111,12 @@ size_t workspace_layout(const lbm_params& p, lbm_ctx* c) {
   const size_t or0 = take((size_t)K * NS * relt);
   const size_t or1 = aa ? or0 : take((size_t)K * NS * relt);
   const size_t osol = take((size_t)N);
-  const size_t onear = take((size_t)N);
-  const size_t olist = take((kWallList + 1) * sizeof(unsigned));
+  // by the shape alone, so that a workspace's size differs between precisions and streaming
+  // modes by what they store
+  const bool walls = p.lattice == LBM_D3Q19 && p.nx <= kPairTX * kPairMaxCluster;
+  const size_t owall = take(walls ? (size_t)((p.nx + kPairTX - 1) / kPairTX) * p.ny * p.nz * 8 : 0);
+  const size_t orow = take(walls ? (size_t)((p.ny + 7) / 8) * p.nz : 0);
+  const size_t ocut = take(walls ? (size_t)(pair_cuts(p) + 1) * sizeof(int) : 0);
   // staging: rho_r, rho_b, momentum/velocity (3), then psi (SC multiphase) or the two
   // multirange Psi_s in the compute type (a seventh row for FP64 storage)
   const int stage_rows = (p.model == LBM_MODEL_SC_MR && p.precision == LBM_FP64) ? 7 : 6;
@@ -129,8 +133,9 @@ size_t workspace_layout(const lbm_params& p, lbm_ctx* c) {
     c->N = N;
     c->px = px;
     c->NS = NS;
-    c->near_wall = c->ws + onear;
-    c->wall_list = reinterpret_cast<unsigned*>(c->ws + olist);
+    c->walls = reinterpret_cast<unsigned long long*>(c->ws + owall);
+    c->rows_walled = c->ws + orow;
+    c->cuts = reinterpret_cast<int*>(c->ws + ocut);
     c->elt = elt;
     c->relt = relt;
     c->aa = aa;
@@ -308,7 +313,7 @@ lbm_status lbm_init_fields(lbm_ctx* c, const double* rho_r, const double* rho_b,
       e = cudaMemcpyAsync(c->solid, solid, N, cudaMemcpyHostToDevice, c->stream);
     }
     c->has_walls = true;
-    if (e == cudaSuccess && lbm::pair_lattice(c->p)) e = lbm::launch_near_wall(c);
+    if (e == cudaSuccess && lbm::pair_lattice(c->p)) e = lbm::launch_wall_words(c);
   } else {
     e = cudaMemsetAsync(c->solid, 0, N, c->stream);
     c->has_walls = false;
@@ -547,7 +552,7 @@ lbm_status lbm_load_state(lbm_ctx* c, const void* src, const uint8_t* solid) {
   if (solid) {
     e = cudaMemcpyAsync(c->solid, solid, N, cudaMemcpyDefault, c->stream);
     c->has_walls = true;
-    if (e == cudaSuccess && lbm::pair_lattice(c->p)) e = lbm::launch_near_wall(c);
+    if (e == cudaSuccess && lbm::pair_lattice(c->p)) e = lbm::launch_wall_words(c);
   } else {
     e = cudaMemsetAsync(c->solid, 0, N, c->stream);
     c->has_walls = false;

@@ -815,22 +815,69 @@ __global__ void __launch_bounds__(kDiagThreads) diag_mr_kernel(const double* __r
   diag_finish<SUMS>(acc, partials, d, cur, a);
 }
 
-// Which nodes are walls or have one beside them, and a list of the latter
-// (lbm_step_pair.cuh).
-__global__ void near_wall_kernel(const uint8_t* __restrict__ solid, uint8_t* __restrict__ near,
-                                 unsigned* __restrict__ list, AuxParams a) {
-  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < a.n; n += (long long)gridDim.x * blockDim.x) {
-    int x, y, z;
-    node_xyz(n, a, x, y, z);
-    bool beside = false;
-#pragma unroll
-    for (int i = 1; i < D3Q19::Q; i++)
-      beside |= solid[wrapped(x + cx<D3Q19>(i), y + cy<D3Q19>(i), z + cz<D3Q19>(i), a)] != 0;
-    near[n] = (solid[n] ? kWallSelf : 0) | (beside ? kWallNear : 0);
-    if (beside && !solid[n]) {
-      const unsigned at = atomicAdd(&list[0], 1u);
-      if (at < kWallList) list[1 + at] = (unsigned)n;
-    }
+// The wall mask as the pair kernel reads it (kWallAny, lbm_step_pair.cuh), one warp per word.
+__global__ void wall_words_kernel(const uint8_t* __restrict__ solid, unsigned long long* __restrict__ words, int tiles,
+                                  AuxParams a) {
+  const int lane = threadIdx.x & 31;
+  const unsigned total = unsigned(tiles) * a.ny * a.nz, warps = gridDim.x * (blockDim.x / 32);
+  for (unsigned w = (blockIdx.x * blockDim.x + threadIdx.x) / 32; w < total; w += warps) {
+    const unsigned row = w / tiles, z = row / a.ny;
+    const int y = int(row - z * a.ny), x = int(w - row * tiles) * 32 - 1 + lane;
+    unsigned lo = 0, hi = 0, any = 0;
+    for (int dz = -1; dz <= 1; dz++)
+      for (int dy = -1; dy <= 2; dy++) {
+        const unsigned Y = unsigned(y + dy + a.ny) % unsigned(a.ny), Z = unsigned(int(z) + dz + a.nz) % unsigned(a.nz);
+        const uint8_t* s = solid + (long long)a.nx * (Y + (long long)a.ny * Z);
+        auto wall = [&](int X) { return X <= a.nx && s[X < 0 ? a.nx - 1 : X < a.nx ? X : 0] != 0; };
+        const unsigned b = __ballot_sync(0xffffffffu, wall(x));
+        const unsigned c = __ballot_sync(0xffffffffu, lane < 2 && wall(x + 32));
+        any |= b | c;
+        if (dz == 0 && dy == 0) {
+          lo = b;
+          hi = c;
+        }
+      }
+    if (lane == 0) words[w] = lo | (unsigned long long)hi << 32 | (any ? kWallAny : 0);
+  }
+}
+
+// The planes of tile rows with walls in sight and the cuts (kWallCost, lbm_step_pair.cuh) of a walled
+// lattice, one block: every thread adds up the costs of its share of the positions, and walks them again from the sum of the threads before.
+constexpr int kCutThreads = 1024;
+__global__ void __launch_bounds__(kCutThreads) wall_cuts_kernel(const unsigned long long* __restrict__ words,
+                                                                uint8_t* __restrict__ rows_walled, int* __restrict__ cuts,
+                                                                int ncuts, int tiles, AuxParams a) {
+  __shared__ long long sums[kCutThreads];
+  const long long total = (long long)((a.ny + 7) / 8) * a.nz;
+  const long long p0 = total * threadIdx.x / kCutThreads, p1 = total * (threadIdx.x + 1) / kCutThreads;
+  auto in_sight = [&](long long pos) {
+    const int row = int(pos / a.nz), z = int(pos - (long long)row * a.nz);
+    unsigned long long any = 0;
+    for (int y = row * 8; y < min(row * 8 + 8, a.ny); y += 2)
+      for (int t = 0; t < tiles; t++) any |= words[((long long)z * a.ny + y) * tiles + t];
+    return (any & kWallAny) != 0;
+  };
+  auto cost = [&](long long pos) { return rows_walled[pos] ? kWallCost : kPlainCost; };
+  long long own = 0;
+  for (long long pos = p0; pos < p1; pos++) {
+    rows_walled[pos] = in_sight(pos);
+    own += cost(pos);
+  }
+  sums[threadIdx.x] = own;
+  for (int off = 1; off < kCutThreads; off *= 2) {
+    __syncthreads();
+    const long long before = (int)threadIdx.x >= off ? sums[threadIdx.x - off] : 0;
+    __syncthreads();
+    sums[threadIdx.x] += before;
+  }
+  __syncthreads();
+  const long long all = sums[kCutThreads - 1];
+  long long sum = sums[threadIdx.x] - own;
+  if (threadIdx.x == 0) cuts[0] = 0;
+  for (long long pos = p0; pos < p1; pos++) {
+    const long long first = sum * ncuts / all + 1;
+    sum += cost(pos);
+    for (long long g = first; g <= sum * ncuts / all; g++) cuts[g] = int(pos + 1);
   }
 }
 
@@ -1028,11 +1075,15 @@ cudaError_t launch_init_eq(lbm_ctx* c, const double* rr, const double* rb, const
   return by_lattice_precision<InitOp>(c, rr, rb, u);
 }
 
-cudaError_t launch_near_wall(lbm_ctx* c) {
-  cudaError_t e = cudaMemsetAsync(c->wall_list, 0, sizeof(unsigned), c->stream);
+cudaError_t launch_wall_words(lbm_ctx* c) {
+  const int tiles = (c->p.nx + kPairTX - 1) / kPairTX;
+  c->launches += 1;
+  wall_words_kernel<<<grid_for((long long)tiles * c->p.ny * c->p.nz, 8, 8192), 256, 0, c->stream>>>(
+      c->solid, c->walls, tiles, aux_params(c));
+  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   c->launches += 1;
-  near_wall_kernel<<<grid_for(c->N, 256, 8192), 256, 0, c->stream>>>(c->solid, c->near_wall, c->wall_list, aux_params(c));
+  wall_cuts_kernel<<<1, kCutThreads, 0, c->stream>>>(c->walls, c->rows_walled, c->cuts, pair_cuts(c->p), tiles, aux_params(c));
   return cudaGetLastError();
 }
 

@@ -39,8 +39,9 @@ struct lbm_ctx {
   bool aa;               // in-place streaming: f[1] == f[0], r[1] == r[0], and cur is the
                          // layout parity of the state (lbm_step_aa.cuh)
   uint8_t* solid;        // [N] wall mask (all zero without walls)
-  uint8_t* near_wall;    // [N] kWallSelf for a wall, kWallNear beside one (pair kernel)
-  unsigned* wall_list;   // the nodes beside a wall (kWallList)
+  unsigned long long* walls;  // the wall mask as the pair kernel reads it (kWallAny)
+  uint8_t* rows_walled;  // [tile rows of 8][nz] whether a plane of a tile row has walls in sight
+  int* cuts;             // [pair_cuts + 1] shares of a walled lattice's work (kWallCost)
   bool has_walls;
   double* stage;         // [6][N] FP64 staging ([7][N] for the multirange model in FP64):
                          // rho_r, rho_b, momentum then u (x, y, z), psi (SC multiphase) or
@@ -99,12 +100,17 @@ inline bool pair_lattice(const lbm_params& p) {
 // elements of the narrowest storage; other lattices are stored densely.
 inline int row_pitch(const lbm_params& p) { return pair_lattice(p) ? (p.nx + 7) / 8 * 8 : p.nx; }
 
+// Cuts of a walled lattice's work: one for each plane of an 8-row tile, up to kMaxCuts.
+inline int pair_cuts(const lbm_params& p) {
+  return (int)std::min<long long>((long long)((p.ny + 7) / 8) * p.nz, kMaxCuts);
+}
+
 // Aux launchers (lbm_aux.cu)
 cudaError_t launch_init_eq(lbm_ctx* c, const double* rr, const double* rb, const double* u);
 // Checkpoint restore in two passes over the populations: accumulate the densities
 // (acc [K][N] FP64), then write deviations relative to them.
-// near_wall and wall_list of the current wall mask.
-cudaError_t launch_near_wall(lbm_ctx* c);
+// c->walls, c->rows_walled and c->cuts from the current wall mask.
+cudaError_t launch_wall_words(lbm_ctx* c);
 cudaError_t launch_restore_accumulate(lbm_ctx* c, const double* plane, int k, double* acc, bool first);
 cudaError_t launch_restore_plane(lbm_ctx* c, const double* plane, int k, int i, const double* acc);
 cudaError_t launch_export_plane(lbm_ctx* c, double* plane, int k, int i);
@@ -149,6 +155,7 @@ StepParams<T> make_step_params(const lbm_ctx* c) {
   s.n = c->N;
   s.px = c->px;
   s.ns = c->NS;
+  s.ncuts = pair_cuts(q);
   double phi[2][3];
   rest_weights(q, phi);
   for (int k = 0; k < 2; k++)

@@ -228,14 +228,13 @@ cudaError_t launch_pair_tile(lbm_ctx* c) {
   // a grid of at most one block per SM leaves room for the next step's blocks beside its own: they
   // come before its last collision (32^3 CG FP32 9.3 -> 8.7 us)
   sp.admit_early = sp.nblk * C <= c->nsm;
-  // the step follows the step before as a programmatic dependent launch, but not between walls:
-  // the waiting blocks of the next kernel then hold up the clusters (101 x 75 x 67: 66 -> 81 us)
-  cfg.numAttrs = FORM == kWalls ? 1 : 2;
+  cfg.numAttrs = 2;  // the step follows the step before as a programmatic dependent launch
   cfg.gridDim = dim3(sp.nblk * C, 1, 1);
   OutArrays<S, RT, ModelTraits<MODEL>::K * L::Q, ModelTraits<MODEL>::K> out;
   for (int a = 0; a < c->K * c->Q; a++) out.f[a] = static_cast<S*>(c->f[c->cur ^ 1]) + a * c->NS;
   for (int k = 0; k < c->K; k++) out.r[k] = static_cast<RT*>(c->r[c->cur ^ 1]) + k * c->NS;
-  return cudaLaunchKernelEx(&cfg, kern, c->tma[c->cur], out, static_cast<const uint8_t*>(c->near_wall),
+  return cudaLaunchKernelEx(&cfg, kern, c->tma[c->cur], out, static_cast<const unsigned long long*>(c->walls),
+                            static_cast<const uint8_t*>(c->rows_walled), static_cast<const int*>(c->cuts),
                             static_cast<const T*>(c->rep_f), &c->diag->status, sp);
 }
 
@@ -244,10 +243,11 @@ cudaError_t launch_pair_tile(lbm_ctx* c) {
 // two blocks of 16 rows, whose halo rows cost 12% of the staging instead of 25% with 8 rows
 // (128^3: 68 us against 73), unless 16 rows do not divide ny or there are fewer such tiles
 // than blocks to hold them (32^3: 10.4 us against 8.8); in 16-bit storage, whose plane
-// buffers are half as large, as four blocks of 8 rows (57.6 against 59.8 us).
+// buffers are half as large, as four blocks of 8 rows (57.6 against 59.8 us), of which three
+// have the registers for walls.
 template <class L, class T, class S, class RT, int MODEL, bool WALLS, bool REP>
 cudaError_t launch_pair_t(lbm_ctx* c) {
-  constexpr int MB = MODEL != kSCMP ? 2 : sizeof(S) == 4 ? 3 : 4;
+  constexpr int MB = MODEL != kSCMP ? 2 : sizeof(S) == 4 || WALLS ? 3 : 4;
   if constexpr (REP) {
     static_assert(!WALLS, "the repulsion force between walls runs on the generic kernel");
     cudaError_t e = launch_rep_prepass_t<L, T, S, RT>(c, c->cur);
@@ -255,15 +255,7 @@ cudaError_t launch_pair_t(lbm_ctx* c) {
     if (c->p.nx % kPairTX != 0 || c->p.ny % 8 != 0) return launch_pair_tile<L, T, S, RT, MODEL, kRagged, 8, MB, true>(c);
     return launch_pair_tile<L, T, S, RT, MODEL, kFull, 8, MB, true>(c);
   } else if constexpr (WALLS) {
-    cudaError_t e = launch_pair_tile<L, T, S, RT, MODEL, kWalls, 8, MB>(c);
-    if (e != cudaSuccess) return e;
-    c->launches += 1;
-    const int grid = (int)std::min<long long>((c->N + 63) / 64, 8LL * c->nsm);
-    wall_step_kernel<L, T, S, RT, MODEL><<<grid, 64, 0, c->stream>>>(
-        static_cast<const S*>(c->f[c->cur]), static_cast<S*>(c->f[c->cur ^ 1]), static_cast<const RT*>(c->r[c->cur]),
-        static_cast<const RT*>(c->r[c->cur ^ 1]), c->solid, c->near_wall, c->wall_list, &c->diag->status,
-        make_step_params<T>(c));
-    return cudaGetLastError();
+    return launch_pair_tile<L, T, S, RT, MODEL, kWalls, 8, MB>(c);
   } else {
     if (c->p.nx % kPairTX != 0 || c->p.ny % 8 != 0) return launch_pair_tile<L, T, S, RT, MODEL, kRagged, 8, MB>(c);
     if constexpr (MODEL == kSCMP && sizeof(S) == 4)

@@ -54,6 +54,7 @@ struct StepParams {
   long long n;            // nodes
   int px;                 // nodes from one stored row to the next
   long long ns;           // elements of a stored array (px * ny * nz)
+  int ncuts;              // entries of the cuts of a walled lattice (lbm_step_pair.cuh)
   int admit_early;        // pair kernel: the next step's blocks may come before the last collision
   T phi[2][3];            // rest-state weights per component and group (CG: Eq. phi; SC: w)
   // CG

@@ -422,12 +422,7 @@ struct PlaneRun {
   int nz, z;
   Segment sg;
   bool valid;
-  __device__ PlaneRun(int b, int nblk, int ncol, int nz_) : nz(nz_) {
-    const long long total = (long long)ncol * nz_;
-    next = total * b / nblk;
-    end = total * (b + 1) / nblk;
-    pop();
-  }
+  __device__ PlaneRun(long long begin, long long end_, int nz_) : next(begin), end(end_), nz(nz_) { pop(); }
   __device__ void pop() {
     valid = next < end;
     if (!valid) return;
@@ -497,10 +492,22 @@ struct OutArrays {
   RT* r[K];
 };
 
-constexpr uint8_t kWallSelf = 1, kWallNear = 2;  // near_wall: a wall node; a neighbour is a wall
-// wall_list: their number, then the nodes beside a wall in any order, if there are at most
-// kWallList of them.
-constexpr unsigned kWallList = 1u << 17;
+// Walls: a 64-bit word for every row of a tile, (z * ny + y) * tiles + tile.  Bit b: column
+// x0 - 1 + b (periodic) is a wall, b = 0 to the tile's width + 1; kWallAny: there is one within
+// rows y - 1 to y + 2 of planes z - 1 to z + 1, all that the nodes of rows y and y + 1 can see.
+constexpr unsigned long long kWallAny = 1ULL << 63;
+// A walled lattice runs two collisions: where a plane of a tile row has walls in sight of any of
+// its nodes, the whole row of tiles (a cluster) takes the one that looks at them, which is half as
+// long again: 128^3 CG FP32 134 us without walls, 149 between two planes, 208 with 15% of the
+// nodes solid at random (SC FP32 65, 75, 101).  One collision for all nodes takes 163 between two
+// planes; a choice by warp 169 and, with single columns of walls, 282 against 195: both
+// collisions together do not fit the instruction cache.  So clusters whose runs are shorter than
+// kShortRun planes, and would change over every few of them, take the walled one throughout (64^3
+// CG FP32 31.5 -> 26.5; the smaller SC code gains at the shortest runs only).
+// Runs are cut by cost: entry g of ncuts + 1 cuts is the (tile row, plane) position before which the
+// share g / ncuts of the work lies, a plane counting kWallCost or kPlainCost.
+constexpr int kPlainCost = 2, kWallCost = 3, kMaxCuts = 16384;
+constexpr int kShortRun = 16, kShortRunSC = 2;
 
 // Forms of the kernel: every tile full (nx % 32 == 0, ny % TY == 0); any size; any size with
 // walls.  The tests for partial tiles cost the full ones 4% (CG 128^3 FP32) to 16% (FP16).
@@ -511,13 +518,14 @@ enum PairForm : int { kFull = 0, kRagged = 1, kWalls = 2 };
 // rows.  Rows are p.px nodes apart (a multiple of 16 bytes, which a tensor map needs), the
 // last tile of a row or column may be partial.  Every index within an array fits 31 bits.
 // REP (colour gradient): the repulsion force rep [3][n] of lbm_rep.cuh is added.
-// With walls (kWalls) the nodes beside one are left to wall_step_kernel, except for their
-// reference densities, which it reads.
+// With walls (kWalls) a wall neighbour's stencil values are the centre's, and what would be
+// pushed into it comes back (halfway bounce-back).
 template <class L, class T, class S, class RT, int MODEL, int FORM, int TY, int MB, bool REP = false>
 __global__ void __launch_bounds__(16 * TY, MB)
     step_kernel_pair(const __grid_constant__ TmaMaps maps,
                      const __grid_constant__ OutArrays<S, RT, ModelTraits<MODEL>::K * L::Q, ModelTraits<MODEL>::K> out,
-                     const uint8_t* __restrict__ near_wall, const T* __restrict__ rep, int* __restrict__ status,
+                     const unsigned long long* __restrict__ walls, const uint8_t* __restrict__ rows_walled,
+                     const int* __restrict__ cuts, const T* __restrict__ rep, int* __restrict__ status,
                      const __grid_constant__ StepParams<T> p) {
   static_assert(sizeof(T) == 4 && sizeof(RT) == 4, "fields are exchanged as 32-bit words");
   static_assert(TY == 8 || TY == 16, "tile rows with a tensor map");
@@ -588,8 +596,17 @@ __global__ void __launch_bounds__(16 * TY, MB)
     }
   };
 
-  PlaneRun ahead(cid, p.nblk, p.ncol, p.nz);  // the next plane to copy
-  PlaneRun cur(cid, p.nblk, p.ncol, p.nz);    // the plane being staged
+  const long long total = (long long)p.ncol * p.nz;
+  // with walls and short runs, every plane takes the walled collision (kShortRun)
+  [[maybe_unused]] const bool one_form = total < (MODEL == kSCMP ? kShortRunSC : kShortRun) * (long long)p.nblk;
+  auto cut = [&](int b) -> long long {  // where run b begins
+    if constexpr (WALLS)
+      if (!one_form) return cuts[(long long)b * p.ncuts / p.nblk];
+    return total * b / p.nblk;
+  };
+  const long long begin = cut(cid), end = cut(cid + 1);
+  PlaneRun ahead(begin, end, p.nz);  // the next plane to copy
+  PlaneRun cur(begin, end, p.nz);    // the plane being staged
   int issued = 0;                              // planes whose copy was issued
   auto issue_next = [&]() {
     if (tid == 0 && alive && ahead.valid) {
@@ -605,6 +622,7 @@ __global__ void __launch_bounds__(16 * TY, MB)
   Comp2 hcs[K];
   int prev_z = 0, prev_y0 = 0;
   int near[2] = {0, 0};
+  [[maybe_unused]] bool walled = false;
   bool prev_interior = false;
 
   for (int J = 0; cur.valid; J++) {
@@ -617,15 +635,35 @@ __global__ void __launch_bounds__(16 * TY, MB)
     const int halo_warp = J % kWarps;  // stages the halo rows too
     const int rows = FULL ? TY : min(TY, p.ny - y0);
     Comp2 cs[K];
-    // what the nodes of plane J are: outside the lattice (as kWallSelf), a wall, beside one
+    // 1: the node is a wall or outside the lattice; otherwise bit i: its neighbour i is a wall
     int next_near[2] = {0, 0};
+    [[maybe_unused]] bool next_walled = false;
+    if constexpr (WALLS) {
+      const int gy = y0 + 2 * warp;
+      next_walled = interior && rows_walled[cur.sg.col * p.nz + z] != 0;
+      if (next_walled && gy < p.ny) {
+        auto word = [&](int y, int zz) { return walls[unsigned(zz * p.ny + y) * unsigned(C) + rank]; };
+        if (word(gy, z) & kWallAny) {
+          unsigned v[3][4];  // columns x-1 .. x+1 of planes z-1 .. z+1, rows gy-1 .. gy+2
+#pragma unroll
+          for (int r = 0; r < 4; r++) {
+            const int y = gy - 1 + r, yw = y < 0 ? p.ny - 1 : y < p.ny ? y : min(y - p.ny, p.ny - 1);
+            v[0][r] = unsigned(word(yw, z == 0 ? p.nz - 1 : z - 1) >> lane);
+            v[1][r] = unsigned(word(yw, z) >> lane);
+            v[2][r] = unsigned(word(yw, z + 1 >= p.nz ? 0 : z + 1) >> lane);
+          }
+#pragma unroll
+          for (int j = 0; j < 2; j++)
+#pragma unroll
+            for (int i = 0; i < Q; i++)
+              next_near[j] |= int((v[cz<L>(i) + 1][cy<L>(i) + 1 + j] >> (cx<L>(i) + 1)) & 1u) << i;
+        }
+      }
+    }
     if constexpr (!FULL) {
 #pragma unroll
-      for (int j = 0; j < 2; j++) {
-        const int gy = y0 + 2 * warp + j;
-        next_near[j] = lane >= width || gy >= p.ny ? kWallSelf : 0;
-        if (WALLS && interior && next_near[j] == 0) next_near[j] = near_wall[x0 + lane + p.nx * (gy + p.ny * z)];
-      }
+      for (int j = 0; j < 2; j++)
+        if (lane >= width || y0 + 2 * warp + j >= p.ny || (next_near[j] & 1)) next_near[j] = 1;
     }
     // ---- stage plane J ----
     if (alive) wait(&raw_full[J % RAW], J / RAW);
@@ -690,7 +728,7 @@ __global__ void __launch_bounds__(16 * TY, MB)
       for (int k = 0; k < 3; k++)
 #pragma unroll
         for (int j = 0; j < 2; j++) {
-          const bool own = prev_interior && (FULL || !(near[j] & kWallSelf));
+          const bool own = prev_interior && (FULL || !(near[j] & 1));
           const unsigned n = x0 + lane + p.nx * (prev_y0 + 2 * warp + j + p.ny * prev_z);
           fr[k].set(j, own ? rep[k * p.n + n] : 0.f);
         }
@@ -726,8 +764,7 @@ __global__ void __launch_bounds__(16 * TY, MB)
     auto ready = [&]() { wait(&fld_full[fs], J / FS); };  // the neighbours' columns of plane J
     if (alive && !prev_interior) ready();
     // ---- collide plane J-1 ----
-    const bool any_live = FULL || __any_sync(0xffffffffu, near[0] == 0 || near[1] == 0 || near[0] == kWallNear ||
-                                                              near[1] == kWallNear);
+    const bool any_live = FULL || __any_sync(0xffffffffu, !(near[0] & near[1] & 1));
     if (alive && prev_interior && !any_live) ready();  // walls, or rows beyond a partial tile
     if (alive && prev_interior && any_live) {
       const int slm = (J + FS - 2) % FS, sl0 = (J + FS - 1) % FS;
@@ -735,10 +772,6 @@ __global__ void __launch_bounds__(16 * TY, MB)
       const float* f_m = fld + slm * NV * NE + e0;
       const float* f_0 = fld + sl0 * NV * NE + e0;
       const float* f_p = fld + fs * NV * NE + e0;
-      auto nb = [&](int f, int i, int j) -> float {
-        const float* base = cz<L>(i) == 0 ? f_0 : (cz<L>(i) > 0 ? f_p : f_m);
-        return base[f * NE + (cy<L>(i) + j) * EX + cx<L>(i)];
-      };
       // storage indices: columns x-1 .. x+1, rows y-1 .. y+2, planes z-1 .. z+1 (periodic)
       const int gx = x0 + lane, gy = prev_y0 + 2 * warp, zz = prev_z;
       auto row = [&](int y) { return unsigned((y >= p.ny ? y - p.ny : y) * p.px); };
@@ -753,35 +786,62 @@ __global__ void __launch_bounds__(16 * TY, MB)
       for (int k = 0; k < K; k++)
 #pragma unroll
         for (int j = 0; j < 2; j++)
-          if (FULL || !(near[j] & kWallSelf)) out.r[k][dest(0, j)] = hcs[k].q[j];
-      // a result of component k, re-referenced to the destination's density (field f), out
-      auto push = [&](int k, int f, int i, const F2& v) {
-        F2 o = v;
-        if (i != 0) {
-          F2 n;
-#pragma unroll
-          for (int j = 0; j < 2; j++) n.set(j, nb(f, i, j));
-          o = fma(F2(p.phi[k][grp<L>(i)]), hcs[k].q - n, v);
-        }
-#pragma unroll
-        for (int j = 0; j < 2; j++)
-          if (FULL || near[j] == 0) out.f[k * Q + i][dest(i, j)] = st_s<S, T>(o[j]);
-      };
-      if constexpr (MODEL == kCG) {
-        auto emit = [&](int i, const F2& vR, const F2& vB) {
-          push(0, 0, i, vR);
-          push(1, 1, i, vB);
+          if (FULL || !(near[j] & 1)) out.r[k][dest(0, j)] = hcs[k].q[j];
+      auto collide = [&](auto with_walls) {
+        constexpr bool WALLED = decltype(with_walls)::value;
+        // field f at neighbour i of node j; at a wall, of the node itself
+        auto nb = [&](int f, int i, int j) -> float {
+          const float* base = cz<L>(i) == 0 ? f_0 : (cz<L>(i) > 0 ? f_p : f_m);
+          const float* at = base + (cy<L>(i) + j) * EX + cx<L>(i);
+          if constexpr (WALLED) at = (near[j] >> i) & 1 ? f_0 + j * EX : at;
+          return at[f * NE];
         };
-        cg_collide_pair<L, REP>(p, hold, hcs[0], hcs[1], fr, nb, ready, emit);
-      } else if constexpr (MODEL == kSC2C) {
-        auto emit = [&](int k, int i, const F2& v) { push(k, k, i, v); };
-        sc2c_collide_pair<L>(p, hold, hcs, nb, ready, emit);
-      } else {
-        F2 psic;
+        // a result of component k, re-referenced to the destination's density (field f), out;
+        // what runs into a wall comes back into the opposite direction's array, ns elements off
+        auto push = [&](int k, int f, int i, const F2& v) {
+          F2 o = v;
+          if (i != 0) {
+            F2 n;
 #pragma unroll
-        for (int j = 0; j < 2; j++) psic.set(j, nb(0, 0, j));
-        auto emit = [&](int i, const F2& v) { push(0, 1, i, v); };
-        scmp_collide_pair<L>(p, hold, hcs[0], psic, nb, ready, emit);
+            for (int j = 0; j < 2; j++) n.set(j, nb(f, i, j));
+            o = fma(F2(p.phi[k][grp<L>(i)]), hcs[k].q - n, v);
+          }
+#pragma unroll
+          for (int j = 0; j < 2; j++) {
+            // (chosen first and stored under one predicate, the walled form takes no branches)
+            int to = int(dest(i, j));
+            if (WALLED && i != 0) {
+              const int back = int(dest(0, j)) + (opp<L>(i) > i ? plane_n * p.nz : -plane_n * p.nz);
+              to = (near[j] >> i) & 1 ? back : to;
+            }
+            S* const at = WALLED ? out.f[k * Q + i] + to : out.f[k * Q + i] + dest(i, j);
+            if (FULL || !(near[j] & 1)) *at = st_s<S, T>(o[j]);
+          }
+        };
+        if constexpr (MODEL == kCG) {
+          auto emit = [&](int i, const F2& vR, const F2& vB) {
+            push(0, 0, i, vR);
+            push(1, 1, i, vB);
+          };
+          cg_collide_pair<L, REP>(p, hold, hcs[0], hcs[1], fr, nb, ready, emit);
+        } else if constexpr (MODEL == kSC2C) {
+          auto emit = [&](int k, int i, const F2& v) { push(k, k, i, v); };
+          sc2c_collide_pair<L>(p, hold, hcs, nb, ready, emit);
+        } else {
+          F2 psic;
+#pragma unroll
+          for (int j = 0; j < 2; j++) psic.set(j, nb(0, 0, j));
+          auto emit = [&](int i, const F2& v) { push(0, 1, i, v); };
+          scmp_collide_pair<L>(p, hold, hcs[0], psic, nb, ready, emit);
+        }
+      };
+      if constexpr (WALLS) {
+        if (walled || one_form)
+          collide(std::true_type{});
+        else
+          collide(std::false_type{});
+      } else {
+        collide(std::false_type{});
       }
     }
     if constexpr (EARLY) {
@@ -802,6 +862,7 @@ __global__ void __launch_bounds__(16 * TY, MB)
     for (int k = 0; k < K; k++) hcs[k] = cs[k];
     near[0] = next_near[0];
     near[1] = next_near[1];
+    walled = next_walled;
     prev_interior = interior;
     prev_z = z;
     prev_y0 = y0;
@@ -813,76 +874,6 @@ __global__ void __launch_bounds__(16 * TY, MB)
     for (int j = max(0, issued - RAW); j < issued; j++) mbar_wait_bounded(&raw_full[j % RAW], (j / RAW) & 1);
   __syncwarp();
   cluster_sync_all();  // no block leaves while a neighbour may still write to it
-}
-
-// The nodes beside a wall, one thread per node, after the pair kernel: the same
-// step with the stencil values of a wall neighbour replaced by the centre's and halfway
-// bounce-back.  The fields are formed from the densities q the pair kernel has written.
-// (Inside the pair kernel the tests for walls of one warp in a tile held up the whole
-// cluster: CG 128 x 72 x 64 between two planes 70 us, 47 without walls.)  The list spares
-// most blocks, of which 255 registers a thread let few run at a time, a look at near_wall:
-// 20 us for the nodes of a 101 x 75 x 67 channel without it.
-template <class L, class T, class S, class RT, int MODEL>
-__global__ void __launch_bounds__(64) wall_step_kernel(
-    const S* __restrict__ fin, S* __restrict__ fout, const RT* __restrict__ rin, const RT* __restrict__ rout,
-    const uint8_t* __restrict__ solid, const uint8_t* __restrict__ near_wall, const unsigned* __restrict__ wall_list,
-    const int* __restrict__ status, const __grid_constant__ StepParams<T> p) {
-  if (*status != 0) return;
-  constexpr int Q = L::Q, K = ModelTraits<MODEL>::K, NF = ModelTraits<MODEL>::NF;
-  const size_t NS = (size_t)p.ns;
-  const unsigned listed = wall_list[0];
-  const bool scan = listed > kWallList;
-  const unsigned count = scan ? (unsigned)p.n : listed;
-  for (unsigned m = blockIdx.x * blockDim.x + threadIdx.x; m < count; m += gridDim.x * blockDim.x) {
-    const int n = scan ? (int)m : (int)wall_list[1 + m];
-    if (scan && near_wall[n] != kWallNear) continue;
-    int x, y, z;
-    node_coords(n, p.nx, p.ny, p.n, x, y, z);
-    const int X[3] = {x == 0 ? p.nx - 1 : x - 1, x, x + 1 >= p.nx ? 0 : x + 1};
-    const int Y[3] = {y == 0 ? p.ny - 1 : y - 1, y, y + 1 >= p.ny ? 0 : y + 1};
-    const int Z[3] = {z == 0 ? p.nz - 1 : z - 1, z, z + 1 >= p.nz ? 0 : z + 1};
-    unsigned to[Q];  // stored index of neighbour i
-    unsigned walls = 0;
-    T fld[NF][Q], q[K][Q], g[K][Q];
-    CompState<T> cs[K];
-#pragma unroll
-    for (int i = 0; i < Q; i++) {
-      const int row = Y[cy<L>(i) + 1] + p.ny * Z[cz<L>(i) + 1];
-      to[i] = X[cx<L>(i) + 1] + p.px * row;
-      walls |= (solid[X[cx<L>(i) + 1] + p.nx * row] ? 1u : 0u) << i;
-#pragma unroll
-      for (int k = 0; k < K; k++) q[k][i] = rout[k * NS + to[i]];
-      T out[2];
-      node_fields<MODEL, T>(p, q[0][i], q[K - 1][i], out);
-#pragma unroll
-      for (int f = 0; f < NF; f++) fld[f][i] = out[f];
-    }
-#pragma unroll
-    for (int k = 0; k < K; k++) {
-#pragma unroll
-      for (int i = 0; i < Q; i++) g[k][i] = ld_s<S, T>(fin[(k * Q + i) * NS + to[0]]);
-      cs[k] = comp_state<L, T, RT>(g[k], rin[k * NS + to[0]]);
-    }
-    auto nbr = [&](int f, int i) -> T { return (walls >> i) & 1u ? fld[f][0] : fld[f][i]; };
-    if constexpr (MODEL == kCG) {
-      const T Fx[3] = {T(0), T(0), T(0)};
-      cg_collide<L, T>(p, g, cs[0], cs[1], nbr, Fx);
-    } else if constexpr (MODEL == kSCMP) {
-      scmp_collide<L, T>(p, g, cs[0], nbr);
-    } else {
-      sc2c_collide<L, T>(p, g, cs[0], cs[1], nbr);
-    }
-#pragma unroll
-    for (int i = 0; i < Q; i++) {
-      const bool bounce = (walls >> i) & 1u;
-#pragma unroll
-      for (int k = 0; k < K; k++) {
-        T v = g[k][i];
-        if (i != 0 && !bounce) v += p.phi[k][grp<L>(i)] * (cs[k].q - q[k][i]);
-        fout[(k * Q + (bounce ? opp<L>(i) : i)) * NS + (bounce ? to[0] : to[i])] = st_s<S, T>(v);
-      }
-    }
-  }
 }
 
 }  // namespace lbm
