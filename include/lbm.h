@@ -176,10 +176,11 @@ const char* lbm_status_string(lbm_status s);
  * The tiling only applies to the generic kernel.  D3Q19 lattices in FP32/FP16/BF16 with two
  * buffers and nx <= 512 run the pair kernel (two nodes per thread), which picks its own
  * shape, except with the repulsion force between walls and, when nx % 32 != 0 or ny % 8 != 0,
- * below 300,000 nodes (600,000 in 16-bit storage with walls) with walls, 16-bit storage or the
- * SC-multiphase model; the generic kernel cuts a lattice with fewer tiles than SMs into smaller
- * ones.  Wider lattices with nx % 32 == 0 and ny % 8 == 0 run a TMA-staged kernel when tx x ty is
- * 32 x 8 (which the 512-node tiles 32 x 16 and 64 x 8 stand for).  Results are
+ * for nx < 12 and, with walls, 16-bit storage or the SC-multiphase model, for nx * ny < 1500
+ * (2000 in 16-bit storage), whatever nz; the generic kernel cuts a lattice with fewer tiles
+ * than SMs into smaller ones.  Wider lattices with nx % 32 == 0 and ny % 8 == 0 run a
+ * TMA-staged kernel when tx x ty is 32 x 8 (which the 512-node tiles 32 x 16 and 64 x 8 stand
+ * for).  Results are
  * bitwise independent of the shape within each kernel; the kernels agree to a few ulps of
  * the stored populations (the compiler fuses multiply-adds differently).  LBM_EINVAL for
  * shapes outside those limits. */

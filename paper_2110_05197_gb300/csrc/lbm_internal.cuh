@@ -7,6 +7,7 @@
 #include <cstdint>
 
 #include "../../include/lbm.h"
+#include "lbm_rules.h"
 #include "lbm_step.cuh"
 #include "lbm_step_pair.cuh"
 #include "lbm_step_tma.cuh"
@@ -88,17 +89,6 @@ size_t step_smem_for(const lbm_ctx* c, int tx, int ty);
 // Encode the tensor maps of both buffer pairs when the lattice suits a TMA-staged kernel:
 // pair_lattice, or D3Q19 in FP32/FP16/BF16 with nx % 32 == 0 and ny % 8 == 0; false otherwise.
 bool build_tma_maps(lbm_ctx* c);
-
-// Whether a lattice is stored for the pair kernel (lbm_step_pair.cuh): D3Q19, 32- or 16-bit
-// storage, two buffers, at most kPairMaxCluster tiles of 32 columns.  (The repulsion force
-// between walls runs elsewhere, on the same storage.)
-inline bool pair_lattice(const lbm_params& p) {
-  return p.lattice == LBM_D3Q19 && p.precision != LBM_FP64 && p.streaming == LBM_STREAM_AB &&
-         p.model != LBM_MODEL_SC_MR && p.nx <= 32 * kPairMaxCluster;
-}
-// Row pitch of the stored arrays: a tensor map needs rows of a multiple of 16 bytes, i.e. 8
-// elements of the narrowest storage; other lattices are stored densely.
-inline int row_pitch(const lbm_params& p) { return pair_lattice(p) ? (p.nx + 7) / 8 * 8 : p.nx; }
 
 // Cuts of a walled lattice's work: one for each plane of an 8-row tile, up to kMaxCuts.
 inline int pair_cuts(const lbm_params& p) {

@@ -265,19 +265,6 @@ cudaError_t launch_pair_t(lbm_ctx* c) {
   }
 }
 
-// Whether the pair kernel steps a lattice.  On aligned ones it is the fastest.  With partial
-// tiles, tuned generic tiles are as fast or faster for the cheap planes of small lattices
-// (61 x 57 x 59: SC FP32 16.6 against 20.7 us, CG FP16 27.0 against 28.9; 75 x 77 x 71: SC FP32
-// 30.9 against 26.8, CG FP16 55.7 against 47.9) and with walls, which cost a second launch
-// (75 x 77 x 71: CG FP32 74.7 against 65.8, FP16 63.8 against 62.0, SC FP16 33.5 against 39.1);
-// FP32 CG and two-component SC without walls gain or are level at every size.
-inline bool pair_steps(const lbm_ctx* c) {
-  if (!c->tma_ok || !pair_lattice(c->p)) return false;
-  const bool aligned = c->p.nx % kPairTX == 0 && c->p.ny % 8 == 0;
-  const bool cheap = c->p.model == LBM_MODEL_SC_MP || c->elt == 2 || c->has_walls;
-  return aligned || !cheap || c->N >= (c->has_walls && c->elt == 2 ? 600000 : 300000);
-}
-
 // Field-pass step (in-place streaming, or the multirange model): the field pass, then the
 // step kernel, both over all nodes.
 template <class L, class T, class S, class RT, int MODEL, bool WALLS, bool REP, class I>
@@ -411,7 +398,7 @@ cudaError_t launch_step_t(lbm_ctx* c) {
   if (c->aa) return launch_fp_t<L, T, S, RT, MODEL, WALLS, REP>(c);
   // the pair kernel, whatever the tiling
   if constexpr (L::D == 3 && sizeof(T) == 4 && !(REP && WALLS))
-    if (pair_steps(c)) return launch_pair_t<L, T, S, RT, MODEL, WALLS, REP>(c);
+    if (c->tma_ok && pair_steps(c->p, WALLS)) return launch_pair_t<L, T, S, RT, MODEL, WALLS, REP>(c);
   if (c->tx * c->ty > 256) {
     // the 512-node tilings run as 32 x 8 persistent tiles
     const int tx = c->tx, ty = c->ty, tz = c->tz;

@@ -42,6 +42,7 @@
 // slots.  Every wait is bounded (lbm_step_tma.cuh).
 #pragma once
 
+#include "lbm_rules.h"
 #include "lbm_step_tma.cuh"
 #include "lbm_vec.cuh"
 
@@ -464,10 +465,8 @@ __device__ __forceinline__ void st_async_f32(uint32_t cluster_addr, float v, uin
                : "memory");
 }
 
-constexpr int kPairTX = 32;
 constexpr int kPairFields = 4;       // field slots
 constexpr int kPairHeader = 128;     // mbarriers, then 128-byte aligned plane buffers
-constexpr int kPairMaxCluster = 16;  // blocks per cluster (the non-portable limit): nx <= 512
 
 template <class L, class S, class RT, int MODEL, int TY>
 __host__ __device__ constexpr size_t pair_smem_bytes(int raw) {

@@ -1,0 +1,40 @@
+"""The rules of csrc/lbm_rules.h, which decide what kernel a lattice runs and how it is stored,
+compiled for the host: z-slabs run the kernel of the whole lattice."""
+import ctypes
+import itertools
+import os
+import subprocess
+
+import pytest
+
+from paper_2110_05197_gb300 import lbm
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SRC = """
+#include "lbm_rules.h"
+extern "C" int pair_steps(const lbm_params* p, int walls) { return lbm::pair_steps(*p, walls != 0); }
+extern "C" int row_pitch(const lbm_params* p) { return lbm::row_pitch(*p); }
+"""
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    d = tmp_path_factory.mktemp("rules")
+    (d / "rules.cpp").write_text(SRC)
+    so = d / "rules.so"
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I",
+                    os.path.join(ROOT, "paper_2110_05197_gb300", "csrc"), str(d / "rules.cpp"), "-o", str(so)], check=True)
+    return ctypes.CDLL(str(so))
+
+
+def _c(**kw):
+    return ctypes.byref(lbm.Params(**kw).to_c())
+
+
+def test_slabs_run_the_kernel_of_the_whole_lattice(rules):
+    for (nx, ny), model, precision, walls in itertools.product(
+            [(8, 200), (33, 33), (61, 57), (97, 75), (101, 75), (64, 64), (200, 203), (512, 40)], (0, 1, 2), (1, 2, 3),
+            (False, True)):
+        kinds = {rules.pair_steps(_c(nx=nx, ny=ny, nz=nz, model=model, precision=precision), walls)
+                 for nz in (4, 17, 60, 67, 300, 1000)}
+        assert len(kinds) == 1, (nx, ny, model, precision, walls)
