@@ -111,9 +111,13 @@ size_t workspace_layout(const lbm_params& p, lbm_ctx* c) {
   const size_t or0 = take((size_t)K * NS * relt);
   const size_t or1 = aa ? or0 : take((size_t)K * NS * relt);
   const size_t osol = take((size_t)N);
-  // by the shape alone, so that a workspace's size differs between precisions and streaming
+  // by the shape alone, so that a workspace's size differs between models, precisions and streaming
   // modes by what they store
-  const bool walls = p.lattice == LBM_D3Q19 && p.nx <= kPairTX * kPairMaxCluster;
+  lbm_params shape = p;
+  shape.model = LBM_MODEL_CG;
+  shape.precision = LBM_FP32;
+  shape.streaming = LBM_STREAM_AB;
+  const bool walls = pair_lattice(shape);
   const size_t owall = take(walls ? (size_t)((p.nx + kPairTX - 1) / kPairTX) * p.ny * p.nz * 8 : 0);
   const size_t orow = take(walls ? (size_t)((p.ny + 7) / 8) * p.nz : 0);
   const size_t ocut = take(walls ? (size_t)(pair_cuts(p) + 1) * sizeof(int) : 0);

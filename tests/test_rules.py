@@ -1,5 +1,6 @@
 """The rules of csrc/lbm_rules.h, which decide what kernel a lattice runs and how it is stored,
-compiled for the host: z-slabs run the kernel of the whole lattice."""
+compiled for the host: z-slabs run the kernel of the whole lattice; rows are padded only where the
+pair kernel reads them, and never beyond what the batched launch takes."""
 import ctypes
 import itertools
 import os
@@ -38,3 +39,20 @@ def test_slabs_run_the_kernel_of_the_whole_lattice(rules):
         kinds = {rules.pair_steps(_c(nx=nx, ny=ny, nz=nz, model=model, precision=precision), walls)
                  for nz in (4, 17, 60, 67, 300, 1000)}
         assert len(kinds) == 1, (nx, ny, model, precision, walls)
+
+
+def test_rows_are_padded_only_for_the_pair_kernel(rules):
+    for nx, ny, model, precision, aa in itertools.product((1, 2, 3, 7, 11, 12, 33, 61, 97, 511, 513), (1, 9, 33, 75),
+                                                          (0, 1, 2, 3), (0, 1, 2), (0, 1)):
+        p = dict(nx=nx, ny=ny, nz=20, model=model, precision=precision, streaming=aa)
+        runs = rules.pair_steps(_c(**p), 0) or rules.pair_steps(_c(**p), 1)
+        assert rules.row_pitch(_c(**p)) == ((nx + 7) // 8 * 8 if runs else nx), p
+
+
+def test_padding_does_not_leave_32_bit_indices(rules):
+    """K Q N below 2^31 and 38 times the padded size above: dense, as the batched launch needs."""
+    n = dict(nx=33, ny=1300, nz=1300)
+    assert 38 * 33 * 1300 ** 2 < 2 ** 31 <= 38 * 40 * 1300 ** 2
+    assert rules.row_pitch(_c(model=0, precision=1, **n)) == 33 and not rules.pair_steps(_c(model=0, precision=1, **n), 0)
+    assert rules.row_pitch(_c(model=1, precision=1, **n)) == 40  # 19 arrays
+    assert rules.row_pitch(_c(model=0, precision=1, nx=33, ny=1400, nz=1400)) == 40  # no batch in any case
