@@ -111,13 +111,13 @@ size_t workspace_layout(const lbm_params& p, lbm_ctx* c) {
   const size_t or0 = take((size_t)K * NS * relt);
   const size_t or1 = aa ? or0 : take((size_t)K * NS * relt);
   const size_t osol = take((size_t)N);
-  // by the shape alone, so that a workspace's size differs between models, precisions and streaming
+  // by the shape, so that a workspace's size differs between models, precisions and streaming
   // modes by what they store
   lbm_params shape = p;
   shape.model = LBM_MODEL_CG;
   shape.precision = LBM_FP32;
   shape.streaming = LBM_STREAM_AB;
-  const bool walls = pair_lattice(shape);
+  const bool walls = pair_lattice(p) || pair_lattice(shape);
   const size_t owall = take(walls ? (size_t)((p.nx + kPairTX - 1) / kPairTX) * p.ny * p.nz * 8 : 0);
   const size_t orow = take(walls ? (size_t)((p.ny + 7) / 8) * p.nz : 0);
   const size_t ocut = take(walls ? (size_t)(pair_cuts(p) + 1) * sizeof(int) : 0);
@@ -317,7 +317,7 @@ lbm_status lbm_init_fields(lbm_ctx* c, const double* rho_r, const double* rho_b,
       e = cudaMemcpyAsync(c->solid, solid, N, cudaMemcpyHostToDevice, c->stream);
     }
     c->has_walls = true;
-    if (e == cudaSuccess && lbm::pair_lattice(c->p)) e = lbm::launch_wall_words(c);
+    if (e == cudaSuccess && lbm::pair_steps(c->p, true)) e = lbm::launch_wall_words(c);
   } else {
     e = cudaMemsetAsync(c->solid, 0, N, c->stream);
     c->has_walls = false;
@@ -556,7 +556,7 @@ lbm_status lbm_load_state(lbm_ctx* c, const void* src, const uint8_t* solid) {
   if (solid) {
     e = cudaMemcpyAsync(c->solid, solid, N, cudaMemcpyDefault, c->stream);
     c->has_walls = true;
-    if (e == cudaSuccess && lbm::pair_lattice(c->p)) e = lbm::launch_wall_words(c);
+    if (e == cudaSuccess && lbm::pair_steps(c->p, true)) e = lbm::launch_wall_words(c);
   } else {
     e = cudaMemsetAsync(c->solid, 0, N, c->stream);
     c->has_walls = false;

@@ -24,12 +24,14 @@ inline int padded_pitch(int nx) { return (nx + 7) / 8 * 8; }
 // z-slabs of a lattice (decomp.py) must run the kernel that the whole lattice runs.
 // Nor are rows padded where that alone would take the arrays beyond 32-bit indices: the batched
 // launch and the generic kernel's 32-bit form take such lattices as long as K Q N < 2^31.
+// The pair kernel's own indices reach over one array in 31 bits, and with walls over two.
 inline bool pair_takes(const lbm_params& p, bool walls) {
   if (p.lattice != LBM_D3Q19 || p.precision == LBM_FP64 || p.streaming != LBM_STREAM_AB ||
       p.model == LBM_MODEL_SC_MR || p.nx > kPairTX * kPairMaxCluster)
     return false;
   const long long rows = (long long)p.ny * p.nz, all = (p.model == LBM_MODEL_SC_MP ? 19 : 38) * rows, limit = 1LL << 31;
   if (all * p.nx < limit && all * padded_pitch(p.nx) >= limit) return false;
+  if (rows * padded_pitch(p.nx) >= (walls ? limit / 2 : limit)) return false;
   if (p.nx % kPairTX == 0 && p.ny % 8 == 0) return true;
   const bool heavy = p.precision == LBM_FP32 && p.model != LBM_MODEL_SC_MP && !walls;
   return p.nx >= 12 && (heavy || (long long)p.nx * p.ny >= (p.precision == LBM_FP32 ? 1500 : 2000));

@@ -56,3 +56,10 @@ def test_padding_does_not_leave_32_bit_indices(rules):
     assert rules.row_pitch(_c(model=0, precision=1, **n)) == 33 and not rules.pair_steps(_c(model=0, precision=1, **n), 0)
     assert rules.row_pitch(_c(model=1, precision=1, **n)) == 40  # 19 arrays
     assert rules.row_pitch(_c(model=0, precision=1, nx=33, ny=1400, nz=1400)) == 40  # no batch in any case
+
+
+def test_lattices_beyond_the_pair_kernels_indices(rules):
+    """One array below 2^31 elements, below 2^30 with walls; 288 GB hold up to 2^31 nodes (SC in FP16)."""
+    for nz, free, walled in ((1000, 1, 1), (1024, 1, 0), (2000, 1, 0), (2048, 0, 0), (2100, 0, 0)):
+        p = dict(nx=512, ny=2048, nz=nz, model=1, precision=2)
+        assert rules.pair_steps(_c(**p), 0) == free and rules.pair_steps(_c(**p), 1) == walled, nz

@@ -22,3 +22,14 @@ def test_workspace_is_what_a_lattice_stores(kw):
     # 64 nodes) and the tiles' wall words (8 bytes for up to 32 nodes, where the shape has them)
     stored = p.n * (buffers * p.ncomp * (p.q * elt + ref) + 1 + 48)
     assert stored <= need.value <= 1.03 * stored + 8192
+
+
+def test_pair_lattices_have_room_for_the_tables_of_walls():
+    """Also where only one component's arrays stay within 32-bit indices (rows padded for SC only)."""
+    lbm_build.build()
+    for model, ncomp in ((lbm.SC_MP, 1), (lbm.CG, 2)):
+        p = lbm.Params(nx=33, ny=1300, nz=1300 if model == lbm.SC_MP else 1400, model=model)
+        need = ctypes.c_size_t(0)
+        assert lbm.lib().lbm_create(ctypes.byref(p.to_c()), None, ctypes.byref(need), None, None) == lbm.OK
+        rows = p.ny * p.nz
+        assert need.value >= 2 * ncomp * 20 * 4 * 40 * rows + 49 * p.n + 2 * 8 * rows + (p.ny + 7) // 8 * p.nz
