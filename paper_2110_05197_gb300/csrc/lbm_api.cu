@@ -280,6 +280,7 @@ lbm_status lbm_create(const lbm_params* p, void* ws, size_t* ws_bytes, void* str
     nsm = 0;
   c->nsm = nsm > 0 ? nsm : 1;
   c->occ_fn = nullptr;
+  c->no_clusters = false;
   c->tma_ok = lbm::build_tma_maps(c);
   *out = c;
   return LBM_OK;

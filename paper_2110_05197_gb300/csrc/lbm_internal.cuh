@@ -62,6 +62,7 @@ struct lbm_ctx {
   bool rep;              // CG repulsion force enabled (rep_pi != 0)
   void* colour;          // [N] rho^N (step compute type), repulsion pre-pass
   void* rep_f;           // [3][N] repulsion force, pre-pass
+  bool no_clusters;      // the pair kernel's clusters do not fit: the generic kernel steps instead
   bool tma_ok;           // tensor maps built: the TMA-staged kernels can run this lattice
   lbm::TmaMaps tma[2];   // maps for reading buffer pair 0 / 1
 };

@@ -217,12 +217,16 @@ cudaError_t launch_pair_tile(lbm_ctx* c) {
   if (c->occ_fn != fn || c->occ_tx != -C) {
     int ncl = 0;
     cfg.gridDim = dim3(C, 1, 1);
-    cudaError_t e = cudaOccupancyMaxActiveClusters(&ncl, kern, &cfg);
-    if (e != cudaSuccess) return e;
+    // a part of a GPU may hold no cluster of this size (its SMs lie in groups of fewer)
+    if (cudaOccupancyMaxActiveClusters(&ncl, kern, &cfg) != cudaSuccess || ncl < 1) {
+      cudaGetLastError();
+      c->no_clusters = true;
+      return cudaErrorNotSupported;
+    }
     c->occ_fn = fn;
     c->occ_tx = -C;
     c->occ_ty = 0;
-    c->occ_blocks = ncl > 0 ? ncl : 1;
+    c->occ_blocks = ncl;
   }
   sp.nblk = (int)std::min<long long>(c->occ_blocks, (long long)sp.ncol * sp.nz);  // clusters
   // a grid of at most one block per SM leaves room for the next step's blocks beside its own: they
@@ -398,7 +402,10 @@ cudaError_t launch_step_t(lbm_ctx* c) {
   if (c->aa) return launch_fp_t<L, T, S, RT, MODEL, WALLS, REP>(c);
   // the pair kernel, whatever the tiling
   if constexpr (L::D == 3 && sizeof(T) == 4 && !(REP && WALLS))
-    if (c->tma_ok && pair_steps(c->p, WALLS)) return launch_pair_t<L, T, S, RT, MODEL, WALLS, REP>(c);
+    if (c->tma_ok && !c->no_clusters && pair_steps(c->p, WALLS)) {
+      const cudaError_t e = launch_pair_t<L, T, S, RT, MODEL, WALLS, REP>(c);
+      if (!c->no_clusters) return e;  // else, from now on, the kernels below
+    }
   if (c->tx * c->ty > 256) {
     // the 512-node tilings run as 32 x 8 persistent tiles
     const int tx = c->tx, ty = c->ty, tz = c->tz;
