@@ -50,9 +50,9 @@ bool is_device_ptr(const void* ptr) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// a pointer that kernels on the current device may write FP64 values through
+// a pointer that kernels on the current device may write through
 bool is_local_ptr(const void* ptr) {
-  if (!ptr || reinterpret_cast<uintptr_t>(ptr) % sizeof(double) != 0) return false;
+  if (!ptr) return false;
   cudaPointerAttributes a;
   int dev = 0;
   if (cudaPointerGetAttributes(&a, ptr) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
@@ -60,6 +60,16 @@ bool is_local_ptr(const void* ptr) {
     return false;
   }
   return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
+// a pinned host pointer, which kernels reach by the same address
+bool is_pinned_ptr(const void* ptr) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, ptr) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeHost && a.devicePointer == ptr;
 }
 
 lbm_status fail(lbm_ctx* c, cudaError_t e) {
@@ -404,7 +414,7 @@ lbm_status lbm_moments(lbm_ctx* c, double* rho_r, double* rho_b, double* u, doub
     const long long len[3] = {N, N, 3 * N};
     bool direct[3], apart = true;
     for (int i = 0; i < 3; i++) {
-      direct[i] = is_local_ptr(given[i]);
+      direct[i] = is_local_ptr(given[i]) && (uintptr_t)given[i] % sizeof(double) == 0;
       for (int k = 0; k < i; k++)
         if (given[i] && given[k])
           apart &= (uintptr_t)(given[i] + len[i]) <= (uintptr_t)given[k] || (uintptr_t)(given[k] + len[k]) <= (uintptr_t)given[i];
@@ -463,18 +473,41 @@ lbm_status lbm_destroy(lbm_ctx* c) {
 uint64_t lbm_launch_count(const lbm_ctx* c) { return c ? c->launches : 0; }
 
 namespace {
-// Copies `rows` rows of nx elements between a stored array (rows c->px apart) and a dense
-// buffer.
-cudaError_t copy_rows(lbm_ctx* c, void* dense, void* stored, size_t rows, size_t elt, bool to_dense) {
-  const size_t w = c->p.nx * elt, pitch = c->px * elt;
-  if (w == pitch)
-    return to_dense ? cudaMemcpyAsync(dense, stored, rows * w, cudaMemcpyDefault, c->stream)
-                    : cudaMemcpyAsync(stored, dense, rows * w, cudaMemcpyDefault, c->stream);
-  return to_dense ? cudaMemcpy2DAsync(dense, w, stored, pitch, w, rows, cudaMemcpyDefault, c->stream)
-                  : cudaMemcpy2DAsync(stored, pitch, dense, w, w, rows, cudaMemcpyDefault, c->stream);
+// Copies `planes` planes of `arrays` stored arrays (NS elements apart, rows c->px apart; the
+// first at `stored`) to or from a dense buffer, array after array.  Padded rows are packed by a
+// kernel, on their way to pageable host memory in the staging area (row by row, the copy engine
+// took 13 ms to load the 81 MB of 101 x 75 x 67 CG FP32 from the host; dense rows take 0.8).
+cudaError_t copy_arrays(lbm_ctx* c, void* dense, void* stored, int arrays, int planes, size_t elt, bool to_dense) {
+  char* const d = static_cast<char*>(dense);
+  char* const st = static_cast<char*>(stored);
+  const size_t per = (size_t)planes * c->p.ny, row = c->p.nx * elt;
+  cudaError_t e = cudaSuccess;
+  if (c->px == c->p.nx) {
+    const bool whole = planes == c->p.nz;
+    const size_t bytes = per * row * (whole ? arrays : 1);
+    for (int a = 0; a < (whole ? 1 : arrays) && e == cudaSuccess; a++) {
+      char* const at = st + a * c->NS * elt;
+      e = to_dense ? cudaMemcpyAsync(d + a * bytes, at, bytes, cudaMemcpyDefault, c->stream)
+                   : cudaMemcpyAsync(at, d + a * bytes, bytes, cudaMemcpyDefault, c->stream);
+    }
+    return e;
+  }
+  const size_t rows = per * arrays;
+  // the kernel reads pinned memory itself (101 x 75 x 67 CG FP32: 0.48 ms, staged 0.56), and writes
+  // what is small (33^3: 72 us, staged 96; large states are staged in 0.53 ms, written in 0.60)
+  const bool direct = is_local_ptr(dense) || (is_pinned_ptr(dense) && (!to_dense || rows * row <= (size_t)8 << 20));
+  if (direct) return lbm::launch_pack_rows(c, dense, stored, 0, rows, per, elt, to_dense);
+  const size_t chunk = (size_t)(6 * c->N) * sizeof(double) / row;
+  for (size_t r = 0; r < rows && e == cudaSuccess; r += chunk) {
+    const size_t n = std::min(chunk, rows - r);
+    if (to_dense) e = lbm::launch_pack_rows(c, c->stage, stored, r, n, per, elt, true);
+    if (e == cudaSuccess)
+      e = to_dense ? cudaMemcpyAsync(d + r * row, c->stage, n * row, cudaMemcpyDefault, c->stream)
+                   : cudaMemcpyAsync(c->stage, d + r * row, n * row, cudaMemcpyDefault, c->stream);
+    if (!to_dense && e == cudaSuccess) e = lbm::launch_pack_rows(c, c->stage, stored, r, n, per, elt, false);
+  }
+  return e;
 }
-// Rows of a whole set of `arrays` stored arrays.
-size_t all_rows(const lbm_ctx* c, int arrays) { return (size_t)arrays * c->p.ny * c->p.nz; }
 }  // namespace
 
 size_t lbm_state_bytes(const lbm_ctx* c) {
@@ -505,9 +538,9 @@ lbm_status lbm_save_state(lbm_ctx* c, void* dst) {
                               c->stream);
       }
   } else {
-    e = copy_rows(c, dst, c->f[b], all_rows(c, c->K * c->Q), c->elt, true);
+    e = copy_arrays(c, dst, c->f[b], c->K * c->Q, c->p.nz, c->elt, true);
   }
-  if (e == cudaSuccess) e = copy_rows(c, static_cast<char*>(dst) + fb, c->r[b], all_rows(c, c->K), c->relt, true);
+  if (e == cudaSuccess) e = copy_arrays(c, static_cast<char*>(dst) + fb, c->r[b], c->K, c->p.nz, c->relt, true);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return fail(c, e);
   return hd.status ? LBM_EUNSTABLE : LBM_OK;
@@ -526,17 +559,11 @@ lbm_status copy_planes(lbm_ctx* c, int32_t z0, int32_t np, void* buf, bool to_bu
   if (!c || !buf || z0 < 0 || np < 1 || z0 + np > c->p.nz) return LBM_EINVAL;
   if (c->sticky != LBM_OK) return c->sticky;
   if (!c->initialised || c->aa) return LBM_ESTATE;
-  const size_t rows = (size_t)np * c->p.ny, first = (size_t)z0 * c->p.ny * c->px;
-  const size_t pb = rows * c->p.nx * c->elt, rb = rows * c->p.nx * c->relt;
-  unsigned char* f = static_cast<unsigned char*>(c->f[c->cur]);
-  unsigned char* r = static_cast<unsigned char*>(c->r[c->cur]);
-  unsigned char* b = static_cast<unsigned char*>(buf);
-  cudaError_t e = cudaSuccess;
-  for (int a = 0; a < c->K * c->Q && e == cudaSuccess; a++)
-    e = copy_rows(c, b + a * pb, f + ((size_t)a * c->NS + first) * c->elt, rows, c->elt, to_buf);
-  for (int k = 0; k < c->K && e == cudaSuccess; k++)
-    e = copy_rows(c, b + (size_t)c->K * c->Q * pb + k * rb, r + ((size_t)k * c->NS + first) * c->relt, rows, c->relt,
-                  to_buf);
+  const size_t first = (size_t)z0 * c->p.ny * c->px, fb = (size_t)np * c->p.ny * c->p.nx * c->K * c->Q * c->elt;
+  cudaError_t e = copy_arrays(c, buf, static_cast<char*>(c->f[c->cur]) + first * c->elt, c->K * c->Q, np, c->elt, to_buf);
+  if (e == cudaSuccess)
+    e = copy_arrays(c, static_cast<char*>(buf) + fb, static_cast<char*>(c->r[c->cur]) + first * c->relt, c->K, np,
+                    c->relt, to_buf);
   return e == cudaSuccess ? LBM_OK : fail(c, e);
 }
 }  // namespace
@@ -564,10 +591,13 @@ lbm_status lbm_load_state(lbm_ctx* c, const void* src, const uint8_t* solid) {
   }
   const size_t fb = (size_t)c->K * c->Q * N * c->elt;
   void* dense = const_cast<void*>(src);
-  for (int b = 0; b < (c->aa ? 1 : 2) && e == cudaSuccess; b++) {
-    e = copy_rows(c, dense, c->f[b], all_rows(c, c->K * c->Q), c->elt, false);
+  if (e == cudaSuccess) e = copy_arrays(c, dense, c->f[0], c->K * c->Q, c->p.nz, c->elt, false);
+  if (e == cudaSuccess) e = copy_arrays(c, static_cast<char*>(dense) + fb, c->r[0], c->K, c->p.nz, c->relt, false);
+  if (!c->aa) {  // the second pair is a copy of the first
     if (e == cudaSuccess)
-      e = copy_rows(c, static_cast<char*>(dense) + fb, c->r[b], all_rows(c, c->K), c->relt, false);
+      e = cudaMemcpyAsync(c->f[1], c->f[0], (size_t)c->K * c->Q * c->NS * c->elt, cudaMemcpyDeviceToDevice, c->stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(c->r[1], c->r[0], (size_t)c->K * c->NS * c->relt, cudaMemcpyDeviceToDevice, c->stream);
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(c->diag, 0, sizeof(lbm_diag), c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);

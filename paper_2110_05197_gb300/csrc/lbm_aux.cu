@@ -881,6 +881,57 @@ __global__ void __launch_bounds__(kCutThreads) wall_cuts_kernel(const unsigned l
   }
 }
 
+// A warp per row, four 32-bit words of it in flight per lane: the stored rows in whole words (their
+// pitch is a multiple of 16 bytes; what lies beyond a row's end is never read), the dense ones in
+// units U of their alignment.  w: units of a dense row; pitch, stride: words of a stored row and array.
+template <class U>
+__global__ void __launch_bounds__(256) pack_rows_kernel(U* __restrict__ dense, unsigned* __restrict__ stored, size_t r0,
+                                                        size_t rows, size_t per, unsigned w, unsigned pitch,
+                                                        size_t stride, bool to_dense) {
+  constexpr unsigned P = 4 / sizeof(U);
+  const unsigned lane = threadIdx.x & 31, words = (w + P - 1) / P;
+  const size_t warps = (size_t)gridDim.x * (blockDim.x / 32);
+  for (size_t r = blockIdx.x * (size_t)(blockDim.x / 32) + threadIdx.x / 32; r < rows; r += warps) {
+    const size_t array = (r0 + r) / per;
+    unsigned* const s = stored + array * stride + (r0 + r - array * per) * pitch;
+    U* const d = dense + r * w;
+    for (unsigned x = lane; x < words; x += 128) {
+      union {
+        unsigned word;
+        U unit[P];
+      } v[4];
+#pragma unroll
+      for (unsigned i = 0; i < 4; i++) {
+        if (x + 32 * i >= words) continue;
+        if (to_dense) v[i].word = s[x + 32 * i];
+        else
+#pragma unroll
+          for (unsigned j = 0; j < P; j++)
+            if ((x + 32 * i) * P + j < w) v[i].unit[j] = d[(x + 32 * i) * P + j];
+      }
+#pragma unroll
+      for (unsigned i = 0; i < 4; i++) {
+        if (x + 32 * i >= words) continue;
+        if (!to_dense) s[x + 32 * i] = v[i].word;
+        else
+#pragma unroll
+          for (unsigned j = 0; j < P; j++)
+            if ((x + 32 * i) * P + j < w) d[(x + 32 * i) * P + j] = v[i].unit[j];
+      }
+    }
+  }
+}
+
+template <class U>
+cudaError_t pack_rows_t(lbm_ctx* c, void* dense, void* stored, size_t r0, size_t rows, size_t per, size_t elt, bool to_dense) {
+  const int blocks = (int)std::min<size_t>((rows + 7) / 8, 8 * (size_t)c->nsm);
+  c->launches += 1;
+  pack_rows_kernel<U><<<blocks, 256, 0, c->stream>>>(static_cast<U*>(dense), static_cast<unsigned*>(stored), r0, rows, per,
+                                                     unsigned(c->p.nx * elt / sizeof(U)), unsigned(c->px * elt / 4),
+                                                     (size_t)c->NS * elt / 4, to_dense);
+  return cudaGetLastError();
+}
+
 int grid_for(long long n, int threads, int cap) {
   long long b = (n + threads - 1) / threads;
   if (b > cap) b = cap;
@@ -1085,6 +1136,15 @@ cudaError_t launch_wall_words(lbm_ctx* c) {
   c->launches += 1;
   wall_cuts_kernel<<<1, kCutThreads, 0, c->stream>>>(c->walls, c->rows_walled, c->cuts, pair_cuts(c->p), tiles, aux_params(c));
   return cudaGetLastError();
+}
+
+// In the largest units that both the elements and the dense buffer's address are multiples of.
+cudaError_t launch_pack_rows(lbm_ctx* c, void* dense, void* stored, size_t r0, size_t rows, size_t per, size_t elt,
+                             bool to_dense) {
+  const size_t units = reinterpret_cast<uintptr_t>(dense) | elt;
+  if (units % 4 == 0) return pack_rows_t<unsigned>(c, dense, stored, r0, rows, per, elt, to_dense);
+  if (units % 2 == 0) return pack_rows_t<unsigned short>(c, dense, stored, r0, rows, per, elt, to_dense);
+  return pack_rows_t<unsigned char>(c, dense, stored, r0, rows, per, elt, to_dense);
 }
 
 cudaError_t launch_restore_accumulate(lbm_ctx* c, const double* plane, int k, double* acc, bool first) {

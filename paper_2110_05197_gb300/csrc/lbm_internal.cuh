@@ -109,6 +109,10 @@ cudaError_t launch_export_all(lbm_ctx* c, double* pops);
 // In-place streaming at odd parity: stored plane (k, i) of the even layout into out [N]
 // (storage type), i.e. slot opp(i) of node x - c_i for every x.
 cudaError_t launch_aa_gather_plane(lbm_ctx* c, void* out, int k, int i);
+// `rows` rows from row r0 on, `per` of them in each of the stored arrays (c->NS elements apart, rows
+// c->px apart, the first at `stored`), to or from dense rows; `dense` is where row r0 goes.
+cudaError_t launch_pack_rows(lbm_ctx* c, void* dense, void* stored, size_t r0, size_t rows, size_t per, size_t elt,
+                             bool to_dense);
 // Densities into rho_r, rho_b (null: the staging area; a single component's rho_b is then
 // left out), velocity into u_out unless that is null, the blow-up status and, if asked for,
 // the totals into the diagnostics record.
