@@ -408,8 +408,9 @@ lbm_status lbm_moments(lbm_ctx* c, double* rho_r, double* rho_b, double* u, doub
   cudaError_t e = cudaSuccess;
   const bool need_diag = rho_r || rho_b || u || totals;
   if (need_diag) {
-    // results go straight to the caller's device buffers, or by way of the staging area; a
-    // device buffer of another GPU, or two that overlap, are filled by copies
+    // results go straight to the caller's device buffers, or by way of the staging area: buffers of
+    // the host or another GPU, ones not aligned to their elements, and densities that overlap
+    // another buffer (their copies come after the velocity) are filled by copies
     const double* given[3] = {rho_r, rho_b, u};
     const long long len[3] = {N, N, 3 * N};
     bool direct[3], apart = true;
@@ -422,7 +423,7 @@ lbm_status lbm_moments(lbm_ctx* c, double* rho_r, double* rho_b, double* u, doub
     double* to[3] = {c->stage, c->stage + N, c->stage + 2 * N};
     if (direct[0] && apart) to[0] = rho_r;
     if (direct[1] && apart) to[1] = rho_b;
-    if (u && is_device_ptr(u)) to[2] = u;
+    if (direct[2]) to[2] = u;
     e = lbm::launch_diagnostics(c, to[0], rho_b || c->K == 2 ? to[1] : nullptr, u ? to[2] : nullptr, totals != nullptr);
     if (e != cudaSuccess) return fail(c, e);
     if (rho_r && to[0] != rho_r) e = copy_out(c, rho_r, to[0], N * sizeof(double), &host);
