@@ -61,9 +61,11 @@ __device__ __forceinline__ Comp2 comp_state2(const F2* g, const F2& r_old) {
   return c;
 }
 
-// Reciprocal within an ulp: the hardware's approximation and one Newton-Raphson step (the
-// IEEE reciprocal's slow-path test and branch cost about 12 instructions a call here, six
-// calls for a pair of nodes).
+// Reciprocal by one Newton-Raphson step, x (2 - a x), from rcp.approx (relative error below 2^-22):
+// within 0.501 ulp for 2^-126 <= |a| <= 2^126, which holds for the densities, viscosities and
+// gradients it is taken of; NaN for 0 and for infinities, which a collision does not survive
+// either way.  Six calls for a pair of nodes: with __frcp_rn in its place 101 x 75 x 67 CG FP32 takes
+// 57.0 us instead of 51.4 and 128^3 with 15% walls 225 instead of 208; 128^3 without walls is level.
 __device__ __forceinline__ float rcp_newton(float a) {
   float x;
   asm("rcp.approx.f32 %0, %1;" : "=f"(x) : "f"(a));
