@@ -185,6 +185,9 @@ const char* lbm_status_string(lbm_status s);
  * the stored populations (the compiler fuses multiply-adds differently).  LBM_EINVAL for
  * shapes outside those limits. */
 lbm_status lbm_set_tiling(lbm_ctx* ctx, int32_t tx, int32_t ty, int32_t tz);
+/* 1 if the step kernel of the lattice, with the walls it has now, takes its shape from
+ * lbm_set_tiling; 0 for those that pick their own (pair kernel, field-pass kernels). */
+int32_t lbm_tiling_used(const lbm_ctx* ctx);
 
 /* ---- Batched stepping -------------------------------------------------------------
  * Many lattices (each an lbm_ctx) advance together: one persistent kernel launch per step

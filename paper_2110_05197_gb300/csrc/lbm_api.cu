@@ -310,6 +310,11 @@ lbm_status lbm_set_tiling(lbm_ctx* c, int32_t tx, int32_t ty, int32_t tz) {
   return LBM_OK;
 }
 
+int32_t lbm_tiling_used(const lbm_ctx* c) {
+  if (!c || c->aa || c->p.model == LBM_MODEL_SC_MR) return 0;
+  return !(c->tma_ok && !c->no_clusters && lbm::pair_steps(c->p, c->has_walls));
+}
+
 lbm_status lbm_init_fields(lbm_ctx* c, const double* rho_r, const double* rho_b, const double* u,
                            const uint8_t* solid, const double* pops) {
   if (!c) return LBM_EINVAL;

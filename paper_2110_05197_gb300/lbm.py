@@ -65,6 +65,7 @@ SIGNATURES = {
     "lbm_destroy": (ctypes.c_int, [_VP]),
     "lbm_status_string": (ctypes.c_char_p, [ctypes.c_int]),
     "lbm_set_tiling": (ctypes.c_int, [_VP, ctypes.c_int32, ctypes.c_int32, ctypes.c_int32]),
+    "lbm_tiling_used": (ctypes.c_int32, [_VP]),
     "lbm_launch_count": (ctypes.c_uint64, [_VP]),
     "lbm_state_bytes": (ctypes.c_size_t, [_VP]),
     "lbm_save_state": (ctypes.c_int, [_VP, _VP]),
@@ -270,6 +271,10 @@ class Lattice:
     def set_tiling(self, tx: int, ty: int, tz: int):
         _check(lib().lbm_set_tiling(self._h, tx, ty, tz), "lbm_set_tiling")
         return self
+
+    def tiling_used(self) -> bool:
+        """Whether the lattice's step kernel takes its shape from set_tiling."""
+        return bool(lib().lbm_tiling_used(self._h))
 
     def init(self, rho_r, rho_b=None, u=None, solid=None, pops=None):
         """Arrays may be torch tensors (device or host) or numpy arrays, FP64 (uint8 for

@@ -1,12 +1,13 @@
 """Launch-shape autotuner for the fused step kernel.
 
 For a lattice it times a handful of tilings (block columns tx x ty, z planes per block tz,
-tz = 0 for the persistent grid; 32 x 8 selects the TMA-staged kernel where the lattice
-allows it) on the lattice's own
+tz = 0 for the persistent grid; on lattices of more than 512 columns 32 x 8 selects the
+TMA-staged kernel where it applies) on the lattice's own
 state, keeps the fastest, and restores the state bit for bit (raw state save/load), so
 tuning never changes a simulation's result.  The choice is cached per lattice shape,
 model, precision, walls and repulsion so that every lattice of a shape runs the same
-kernel (results then do not depend on what else was tuned or batched).
+kernel (results then do not depend on what else was tuned or batched).  A lattice whose kernel
+picks its own shape (Lattice.tiling_used) has one candidate, the default.
 """
 from __future__ import annotations
 
@@ -64,7 +65,10 @@ def autotune(lat: "lbm.Lattice", candidates=None, steps: int = 10, trials: int =
     state = lat.save_state()
     solid = getattr(lat, "_solid", None)
     timings = {}
-    for t in (candidates or candidates_for(lat.params)):
+    if candidates is None:
+        p = lat.params
+        candidates = candidates_for(p) if lat.tiling_used() else [(32, 8, min(16, p.nz))]
+    for t in candidates:
         try:
             lat.set_tiling(*t)
         except lbm.LbmError:
