@@ -3,14 +3,15 @@
 // multiphase and two-component models; any nx up to 512, any ny and nz, walls).
 //
 // Same step and densities as the other step kernels (lbm_step.cuh); what differs is the
-// work per instruction.  The step is bound by issued instructions rather than bytes (a
-// one-node-per-thread version of this structure issued 848 (Shan-Chen) to 1403 (colour
+// work per instruction.  One node per thread, this structure issued 848 (Shan-Chen) to 1403 (colour
 // gradient) instructions per node, at 43-58% of the issue slots, with DRAM at 46% of its
-// peak), so both nodes' FP32 arithmetic runs as packed f32x2 instructions (lbm_vec.cuh), the
+// peak: both nodes' FP32 arithmetic runs as packed f32x2 instructions (lbm_vec.cuh), the
 // collision is written with the fewest operations (below), and a store address is one
-// multiply-add of a constant base and a 32-bit node index.  That is 430 (SC) and 750 (CG)
-// instructions per node.  At 128^3: CG FP32 177 -> 137 us, SC FP32 84 -> 68 us, SC FP16
-// 82 -> 58 us; at 256^3 CG FP32 runs at 5.2 TB/s of algorithmic bytes.
+// multiply-add of a constant base and a 32-bit node index.  That is 474 (SC) and 745 (CG)
+// instructions per node at 41% and 32% of the issue slots, with DRAM at 56% and 68%: what is left
+// above the bytes is the latency of a plane's chain (copy, fields, barrier, neighbours' columns,
+// collision, stores) with 16 and 8 warps per SM to hide it.  At 128^3: CG FP32 177 -> 135 us, SC
+// FP32 84 -> 65 us, SC FP16 82 -> 57 us; at 256^3 CG FP32 runs at 5.2 TB/s of algorithmic bytes.
 //
 // Per plane J of a block's sequence, every thread
 //   1. reads its two nodes of plane J from the raw plane buffer (a TMA copy of the tile's
@@ -630,7 +631,7 @@ __global__ void __launch_bounds__(16 * TY, MB)
     const int y0 = cur.sg.col * TY;
     const int z = cur.z;
     const bool interior = z >= cur.sg.z0 && z < cur.sg.z1;  // plane J is collided in iteration J+1
-    if (p.admit_early && cur.last()) admit_next_step();
+    if (!REP && p.admit_early && cur.last()) admit_next_step();
     const int fs = J % FS;
     const unsigned char* b = bufs + (J % RAW) * Lay::BUF_MAIN;
     const int halo_warp = J % kWarps;  // stages the halo rows too
@@ -869,7 +870,7 @@ __global__ void __launch_bounds__(16 * TY, MB)
     prev_y0 = y0;
     cur.advance();
   }
-  admit_next_step();
+  if (!REP) admit_next_step();  // (a plain launch follows: the next step's force)
   // the copies this block issued have landed before its shared memory is released
   if (tid == 0)
     for (int j = max(0, issued - RAW); j < issued; j++) mbar_wait_bounded(&raw_full[j % RAW], (j / RAW) & 1);
